@@ -227,7 +227,9 @@ PF_API pf_status pf_filter_plain_exact(pf_ctx *ctx, unsigned deciders, const pf_
  * number of configurations into *count.  The two-phase form builds every
  * word's mask words (and runs GateKeeper) first, then runs SneakySnake as a
  * per-thread loop of steps over them; longer pairs, and GateKeeper alone,
- * take the fused word loop. */
+ * take the fused word loop.  An exact-threshold configuration with more than
+ * one lane is bit-sliced: its lanes share 32 pairs, one bit of each word per
+ * pair, and split the diagonals among them. */
 PF_API pf_status pf_kernel_configs(int *tpp, int *dpt, int *ecap, int *exact_e, int *words,
                                    int cap, int *count);
 

@@ -519,7 +519,8 @@ def pf_kernel_configs():
     """List of (tpp, dpt, ecap, exact_e, words) of the batch scheduler's
     kernels; exact_e >= 0 marks a kernel that serves that threshold only,
     words > 0 its two-phase form (mask words of pairs up to that many
-    32-column words kept in shared memory)."""
+    32-column words kept in shared memory), exact_e >= 0 with tpp > 1 a
+    bit-sliced one (tpp lanes share 32 pairs)."""
     import numpy as np
     cnt = ctypes.c_int()
     _check(load().pf_kernel_configs(None, None, None, None, None, 0, ctypes.byref(cnt)))

@@ -280,28 +280,26 @@ int pf_ctx::grid_for(int dec, int cfg) {
     return g;
 }
 
-// Default configuration for threshold E before any tuning: the
-// exact-threshold one-thread kernel up to E = 15 (its two-phase form for
-// E = 1..7, with shared arrays that hold pairs up to 256 bases), eight
-// lanes per pair above (the two-phase lane-group form: at 250 bp, E = 25 it
-// takes 3.26 ms per 2M pairs with both deciders against 3.74 for the fused
-// loop).
-int pf::pf_default_cfg(int E) {
+// Default configuration for threshold E before any tuning.  The bit-sliced
+// kernels from the threshold on at which their fixed cost (transposing the
+// planes) is less than what they save per diagonal.  Measured at 100, 150 and
+// 250 bp (4M, 4M, 2M pairs; ms, best word-per-pair kernel -> bit-sliced):
+// SneakySnake alone E = 5 0.24 -> 0.22, 0.28 -> 0.28, (E = 4) 0.24 -> 0.26; E = 6
+// (150, 250) 0.31 -> 0.29, 0.29 -> 0.26; both deciders E = 5 0.32 -> 0.26,
+// 0.37 -> 0.33, (E = 4) 0.24 -> 0.29, (E = 6) 0.34 -> 0.33; GateKeeper alone, which
+// has no walk to save, E = 8 0.28 -> 0.26, 0.33 -> 0.34, 0.26 -> 0.32, E = 15
+// (150) 0.58 -> 0.46.  Below, the exact-threshold one-thread kernel (its
+// two-phase form for E = 1..7, with shared arrays that hold pairs up to 256
+// bases).
+int pf::pf_default_cfg(int dec, int E) {
+    const int sliced_from = dec == 2 ? 12 : (dec == 1 ? 6 : 5);
+    if (E >= sliced_from)
+        for (int c = 0; c < kNumBatchCfgs; ++c)
+            if (kBatchCfgs[c].xe == E && cfg_sliced(kBatchCfgs[c])) return c;
     if (E >= 1 && E <= 7)
         for (int c = 0; c < kNumBatchCfgs; ++c)
             if (kBatchCfgs[c].xe == E && kBatchCfgs[c].words >= 8) return c;
-    if (E <= 15) return kFirstExactCfg + E;
-    // the two-phase form with two or four lanes per pair and the fewest
-    // slots that hold the 2E+1 diagonals (four lanes on a tie)
-    int best = -1;
-    for (int c = 0; c < kNumBatchCfgs; ++c) {
-        const KernelCfg &k = kBatchCfgs[c];
-        if ((k.tpp != 2 && k.tpp != 4) || k.xe >= 0 || k.ecap < E || k.words < 8) continue;
-        if (best < 0 || k.ecap < kBatchCfgs[best].ecap ||
-            (k.ecap == kBatchCfgs[best].ecap && k.tpp > kBatchCfgs[best].tpp))
-            best = c;
-    }
-    return best;
+    return kFirstExactCfg + E;
 }
 
 // E = 0 compares one diagonal and is bound by memory: the plain kernel
@@ -311,7 +309,7 @@ static bool default_plain(int E) { return E == 0; }
 void pf_ctx::reset_tuning() {
     for (int d = 0; d < 4; ++d)
         for (int e = 0; e <= PF_MAX_E; ++e) {
-            tune_cfg[d][e] = pf_default_cfg(e);
+            tune_cfg[d][e] = pf_default_cfg(d, e);
             tune_chunk[d][e] = 256;
             tune_plain[d][e] = default_plain(e);
         }

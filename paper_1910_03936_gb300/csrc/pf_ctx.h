@@ -24,7 +24,7 @@ struct ServeState;
 
 constexpr int kSideStreams = 4;
 
-int pf_default_cfg(int E);
+int pf_default_cfg(int dec, int E);
 
 }  // namespace pf
 

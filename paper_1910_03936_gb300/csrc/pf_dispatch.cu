@@ -16,6 +16,37 @@ cudaError_t launch_plain_exact_dec1(int, const FilterArgs &, cudaStream_t);
 cudaError_t launch_plain_exact_dec2(int, const FilterArgs &, cudaStream_t);
 cudaError_t launch_plain_exact_dec3(int, const FilterArgs &, cudaStream_t);
 
+cudaError_t launch_sliced_1(int, int, const BatchArgs &, int, cudaStream_t);
+cudaError_t launch_sliced_5(int, int, const BatchArgs &, int, cudaStream_t);
+cudaError_t launch_sliced_6(int, int, const BatchArgs &, int, cudaStream_t);
+cudaError_t launch_sliced_7(int, int, const BatchArgs &, int, cudaStream_t);
+const void *sliced_ptr_1(int);
+const void *sliced_ptr_6(int);
+const void *sliced_ptr_7(int);
+
+// SneakySnake alone counts the Hamming distance only for a caller that
+// resolves distances by it.
+cudaError_t launch_filter_sliced(int dec, int cfg, int grid, const BatchArgs &b, int bin,
+                                 cudaStream_t st) {
+    switch (dec) {
+        case 1:
+            return b.f.need ? launch_sliced_5(cfg, grid, b, bin, st)
+                            : launch_sliced_1(cfg, grid, b, bin, st);
+        case 2: return launch_sliced_6(cfg, grid, b, bin, st);
+        case 3: return launch_sliced_7(cfg, grid, b, bin, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+const void *filter_sliced_fn(int dec, int cfg) {
+    switch (dec) {
+        case 1: return sliced_ptr_1(cfg);
+        case 2: return sliced_ptr_6(cfg);
+        case 3: return sliced_ptr_7(cfg);
+    }
+    return nullptr;
+}
+
 cudaError_t launch_filter_plain_exact(int dec, int E, const FilterArgs &a, cudaStream_t st) {
     switch (dec) {
         case 1: return launch_plain_exact_dec1(E, a, st);
@@ -36,6 +67,7 @@ cudaError_t launch_filter_plain(int dec, int plain_idx, const FilterArgs &a, cud
 
 cudaError_t launch_filter_batched(int dec, int cfg, int grid, const BatchArgs &b, int bin,
                                   cudaStream_t st) {
+    if (cfg_sliced(kBatchCfgs[cfg])) return launch_filter_sliced(dec, cfg, grid, b, bin, st);
     switch (dec) {
         case 1: return launch_batched_dec1(cfg, grid, b, bin, st);
         case 2: return launch_batched_dec2(cfg, grid, b, bin, st);
@@ -45,6 +77,7 @@ cudaError_t launch_filter_batched(int dec, int cfg, int grid, const BatchArgs &b
 }
 
 const void *filter_batched_fn(int dec, int cfg) {
+    if (cfg_sliced(kBatchCfgs[cfg])) return filter_sliced_fn(dec, cfg);
     switch (dec) {
         case 1: return batched_fn_dec1(cfg);
         case 2: return batched_fn_dec2(cfg);

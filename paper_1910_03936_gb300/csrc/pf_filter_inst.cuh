@@ -61,14 +61,16 @@ static cudaError_t launch_batched_i(int grid, const BatchArgs &b, int bin, cudaS
 template <int I>
 static cudaError_t launch_batched_r(int cfg, int grid, const BatchArgs &b, int bin,
                                     cudaStream_t st) {
-    if (cfg == I) return launch_batched_i<I>(grid, b, bin, st);
+    if constexpr (!cfg_sliced(kBatchCfgs[I]))
+        if (cfg == I) return launch_batched_i<I>(grid, b, bin, st);
     if constexpr (I + 1 < kNumBatchCfgs) return launch_batched_r<I + 1>(cfg, grid, b, bin, st);
     return cudaErrorInvalidValue;
 }
 
 template <int I>
 static const void *batched_ptr_r(int cfg) {
-    if (cfg == I) return batched_ptr_i<I>();
+    if constexpr (!cfg_sliced(kBatchCfgs[I]))
+        if (cfg == I) return batched_ptr_i<I>();
     if constexpr (I + 1 < kNumBatchCfgs) return batched_ptr_r<I + 1>(cfg);
     return nullptr;
 }

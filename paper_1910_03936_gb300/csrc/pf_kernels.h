@@ -14,8 +14,11 @@ namespace pf {
 // > 0 marks its two-phase form: the mask words of pairs up to `words`
 // 32-column words are kept in shared memory and SneakySnake runs as a
 // per-lane step loop over them (longer pairs take the fused loop).
+// sliced marks a bit-sliced configuration (pf_sliced.cuh): tpp lanes share 32
+// pairs of threshold xe with dpt diagonals each.
 struct KernelCfg {
     int tpp, dpt, ecap, xe, words;
+    bool sliced = false;
 };
 
 constexpr KernelCfg kBatchCfgs[] = {
@@ -54,7 +57,34 @@ constexpr KernelCfg kBatchCfgs[] = {
     // lane groups of two and four (fewer shuffles per step, the walk's
     // control repeated by fewer lanes): the fastest at E = 16..31
     {2, 17, 16, -1, 8},  {4, 11, 21, -1, 8},  {4, 13, 25, -1, 8},  {2, 26, 25, -1, 8},
+    // bit-sliced, one threshold each: E = 5..27 with four lanes per group (at
+    // E = 20 and 25 eight lanes were no faster: 0.54 against 0.52 and 0.63
+    // against 0.57 ms per 2M pairs of 250 bp with both deciders), E = 28..31
+    // with eight (more diagonals per lane than registers hold)
+    {4, 3, 5, 5, 0, true}, {4, 4, 6, 6, 0, true}, {4, 4, 7, 7, 0, true},
+    {4, 5, 8, 8, 0, true}, {4, 5, 9, 9, 0, true}, {4, 6, 10, 10, 0, true},
+    {4, 6, 11, 11, 0, true}, {4, 7, 12, 12, 0, true}, {4, 7, 13, 13, 0, true},
+    {4, 8, 14, 14, 0, true}, {4, 8, 15, 15, 0, true}, {4, 9, 16, 16, 0, true},
+    {4, 9, 17, 17, 0, true}, {4, 10, 18, 18, 0, true}, {4, 10, 19, 19, 0, true},
+    {4, 11, 20, 20, 0, true}, {4, 11, 21, 21, 0, true}, {4, 12, 22, 22, 0, true},
+    {4, 12, 23, 23, 0, true}, {4, 13, 24, 24, 0, true}, {4, 13, 25, 25, 0, true},
+    {4, 14, 26, 26, 0, true}, {4, 14, 27, 27, 0, true}, {8, 8, 28, 28, 0, true},
+    {8, 8, 29, 29, 0, true}, {8, 8, 30, 30, 0, true}, {8, 8, 31, 31, 0, true},
 };
+
+constexpr bool cfg_sliced(const KernelCfg &c) { return c.sliced; }
+
+// A bit-sliced warp's tile: columns per block of the walk, words per segment
+// and words of shared memory (SliceColumns).
+__host__ __device__ constexpr int slice_block(int L) { return L == 8 ? 8 : 4; }
+__host__ __device__ constexpr int slice_seg(int L) { return L / 4; }
+__host__ __device__ constexpr size_t slice_smem_words(int L) {
+    return (size_t)3 * (32 / L) * (32 * (slice_seg(L) + 2) + slice_block(L) - 1 + 32 * slice_seg(L));
+}
+// Warps per SM that a kernel's registers are held to: 168 each, or 255 where
+// the diagonals of a lane need them (GateKeeper also keeps four columns of
+// each).  At 128 registers (16 warps) the kernels were no faster.
+constexpr int slice_warps(int DPT, bool gatekeeper) { return DPT <= (gatekeeper ? 6 : 8) ? 12 : 8; }
 
 // The two-phase form applies where SneakySnake runs (deciders 1 and 3);
 // GateKeeper alone runs a two-phase configuration as the fused loop.
@@ -63,9 +93,10 @@ constexpr bool cfg_split(const KernelCfg &c, int dec) { return c.words > 0 && de
 constexpr int cfg_slots(const KernelCfg &c) { return c.xe >= 0 ? 2 * c.xe + 1 : c.dpt; }
 // Block size and dynamic shared memory of a configuration's kernel.
 constexpr int cfg_threads(const KernelCfg &c, int dec) {
-    return cfg_split(c, dec) ? kSplitWarps * 32 : 256;
+    return cfg_sliced(c) ? 32 : (cfg_split(c, dec) ? kSplitWarps * 32 : 256);
 }
 constexpr size_t cfg_smem(const KernelCfg &c, int dec) {
+    if (cfg_sliced(c)) return slice_smem_words(c.tpp) * sizeof(uint32_t);
     return cfg_split(c, dec)
                ? (size_t)kSplitWarps * c.words * cfg_slots(c) * 32 * sizeof(uint32_t)
                : 0;
@@ -73,7 +104,9 @@ constexpr size_t cfg_smem(const KernelCfg &c, int dec) {
 
 // Pairs one warp of a configuration's kernel takes at once: one per lane in
 // the two-phase form, one per lane group in the fused loop.
-constexpr int cfg_step(const KernelCfg &c, int dec) { return 32 / c.tpp; }
+constexpr int cfg_step(const KernelCfg &c, int dec) {
+    return cfg_sliced(c) ? 32 * (32 / c.tpp) : 32 / c.tpp;
+}
 
 // a configuration serves threshold E
 constexpr bool cfg_serves(const KernelCfg &c, int E) {
@@ -103,6 +136,9 @@ cudaError_t launch_filter_plain_exact(int dec, int E, const FilterArgs &a, cudaS
 cudaError_t launch_filter_batched(int dec, int cfg, int grid, const BatchArgs &b, int bin,
                                   cudaStream_t st);
 const void *filter_batched_fn(int dec, int cfg);
+cudaError_t launch_filter_sliced(int dec, int cfg, int grid, const BatchArgs &b, int bin,
+                                 cudaStream_t st);
+const void *filter_sliced_fn(int dec, int cfg);
 
 cudaError_t launch_pack_ragged(const uint8_t *ascii, const int64_t *byte_off,
                                const int64_t *word_off, int64_t nseq, uint32_t *lo,

@@ -1,0 +1,156 @@
+"""The bit-sliced kernels at the edges of their tiles, against the oracle:
+ragged pairs of mixed lengths in one tile, lengths around word and segment
+boundaries, bins of fewer pairs than a tile, words in any order, planes of
+different layouts on the two sides, and invalid per-pair thresholds."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pf():
+    from paper_1910_03936_gb300 import build
+    build.build()
+    import paper_1910_03936_gb300 as m
+    return m
+
+
+@pytest.fixture()
+def ctx(pf):
+    c = pf.pf_create(0)
+    pf.pf_set_small_batch(c, 0)
+    # every threshold that a bit-sliced configuration serves
+    cfgs = pf.pf_kernel_configs()
+    for e in range(32):
+        own = [i for i, x in enumerate(cfgs) if x[3] == e and x[0] > 1]
+        for dec in (1, 2, 3):
+            if own:
+                pf.pf_tune_set(c, dec, e, own[0], 64)
+    yield c
+    pf.pf_destroy(c)
+
+
+def ragged(seed, lens, E, kmax=40):
+    """Pairs of the given lengths and thresholds with N's, random edits and
+    some reads that match nowhere."""
+    rng = np.random.default_rng(seed)
+    off = np.zeros(len(lens) + 1, dtype=np.int64)
+    np.cumsum(lens, out=off[1:])
+    letters = np.frombuffer(b"ACGTN", np.uint8)
+    prob = [0.295, 0.205, 0.205, 0.29, 0.005]
+    refs = rng.choice(letters, size=max(int(off[-1]), 1), p=prob)
+    reads = refs.copy()
+    for p, m in enumerate(lens):
+        r = list(refs[off[p]:off[p] + m])
+        for _ in range(int(rng.integers(0, min(kmax, 2 * E[p] + 3)))):
+            at = int(rng.integers(0, m)) if m else 0
+            kind = rng.integers(0, 3)
+            if not m:
+                break
+            if kind == 0:
+                r[at] = rng.choice(letters)
+            elif kind == 1:
+                r.insert(at, rng.choice(letters))
+            else:
+                del r[at]
+                r.append(rng.choice(letters))
+        reads[off[p]:off[p] + m] = np.array(r[:m], np.uint8)
+    return synth.Pairs(reads[:off[-1]], refs[:off[-1]], off, off,
+                       np.asarray(lens, np.int32), np.asarray(E, np.int16))
+
+
+def check(pf, ctx, P, pairs, E, E_max, bad=()):
+    dev = "cuda:0"
+    n = P.n
+    oa, oc = oracle.filter_batch(P)
+    od = oracle.verify_batch(P)
+    ok = np.ones(n, bool)
+    ok[list(bad)] = False
+    lens = torch.from_numpy(P.lens).to(dev)
+    Ed = None if E is None else torch.from_numpy(np.asarray(E, np.int16)).to(dev)
+    for dec in (1, 2, 3):
+        slots = 2 if dec == 3 else 1
+        rows = [0, 1] if dec == 3 else [dec - 1]
+        acc = torch.full((slots * n,), 9, dtype=torch.uint8, device=dev)
+        cnt = torch.full((slots * n,), 99, dtype=torch.int16, device=dev)
+        dist = torch.full((n,), -7, dtype=torch.int32, device=dev)
+        pf.pf_filter_verify(ctx, dec, pairs, lens, Ed, E_max, acc, cnt, dist, n)
+        if len(bad):
+            with pytest.raises(pf.PFError):
+                pf.pf_sync(ctx)
+        else:
+            pf.pf_sync(ctx)
+        c = cnt.cpu().numpy().reshape(slots, n)
+        a = acc.cpu().numpy().reshape(slots, n)
+        assert np.array_equal(c[:, ok], oc[rows][:, ok])
+        assert np.array_equal(a[:, ok], oa[rows][:, ok])
+        want = np.where(oa[rows[0]] == 1, od, P.E.astype(np.int32) + 1)
+        assert np.array_equal(dist.cpu().numpy()[ok], want[ok])
+        assert (c[:, ~ok] == -1).all() and (a[:, ~ok] == 0).all()
+        assert (dist.cpu().numpy()[~ok] == -1).all()
+
+
+@pytest.mark.parametrize("E", [5, 7, 11, 16, 27, 28, 31])
+@pytest.mark.parametrize("n", [1, 255, 257, 700])
+def test_lengths_around_words_in_one_tile(pf, ctx, E, n):
+    """One threshold, lengths 0..330 mixed in every tile (pair order: one
+    bin), so that a tile's pairs end in different words and segments."""
+    rng = np.random.default_rng(1000 * E + n)
+    lens = rng.choice([0, 1, 31, 32, 33, 63, 64, 65, 96, 127, 128, 129, 150, 160, 161, 192, 250,
+                       256, 257, 288, 330], size=n)
+    P = ragged(E + n, lens, np.full(n, E))
+    dev = "cuda:0"
+    reads, refs = (torch.from_numpy(np.ascontiguousarray(x if x.size else np.zeros(1, np.uint8))).to(dev)
+                   for x in (P.reads, P.refs))
+    check(pf, ctx, P, pf.pack_pairs(ctx, reads, refs, byte_off=P.read_off), None, E)
+
+
+@pytest.mark.parametrize("m", [1, 32, 150, 160, 250, 256, 300])
+def test_one_length_in_a_strided_layout(pf, ctx, m):
+    """The strided layout (rows of one stride), a last tile of few pairs."""
+    for E in (6, 13, 30):
+        n = 256 * 3 + 41
+        P = ragged(m + E, np.full(n, m), np.full(n, E))
+        dev = "cuda:0"
+        pairs = pf.pack_pairs(ctx, torch.from_numpy(P.reads).to(dev),
+                              torch.from_numpy(P.refs).to(dev), length=m)
+        check(pf, ctx, P, pairs, None, E)
+
+
+@pytest.mark.parametrize("group", [False, True])
+def test_thresholds_and_invalid_pairs_mixed(pf, ctx, group):
+    """Per-pair thresholds 0..31 in bins of some tens of pairs, in both
+    ragged layouts; thresholds above E_max and below 0 are refused pair by
+    pair."""
+    rng = np.random.default_rng(77)
+    n = 3000
+    lens = rng.choice([40, 100, 150, 250], size=n)
+    E = rng.integers(0, 32, size=n)
+    P = ragged(5, lens, E)
+    dev = "cuda:0"
+    reads, refs = torch.from_numpy(P.reads).to(dev), torch.from_numpy(P.refs).to(dev)
+    pairs = pf.pack_pairs(ctx, reads, refs, byte_off=P.read_off, group_E=E if group else None)
+    check(pf, ctx, P, pairs, E, 31)
+    bad = [0, 255, 256, 1700, n - 1]
+    Eb = E.copy()
+    Eb[bad] = [-1, 33, 400, -32768, 32]
+    check(pf, ctx, P, pairs, Eb, 31, bad)
+
+
+def test_sides_in_different_layouts(pf, ctx):
+    """Reads in pair order, references in the grouped layout."""
+    rng = np.random.default_rng(8)
+    n = 900
+    lens = rng.choice([100, 150, 250], size=n)
+    E = rng.integers(5, 26, size=n)
+    P = ragged(6, lens, E)
+    dev = "cuda:0"
+    reads, refs = torch.from_numpy(P.reads).to(dev), torch.from_numpy(P.refs).to(dev)
+    a = pf.pack_pairs(ctx, reads, refs, byte_off=P.read_off)
+    b = pf.pack_pairs(ctx, reads, refs, byte_off=P.read_off, group_E=E)
+    check(pf, ctx, P, pf.Pairs(a.read, b.ref), E, 25)
