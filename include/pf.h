@@ -189,9 +189,10 @@ PF_API pf_status pf_pack_fixed(pf_ctx *ctx, const uint8_t *ascii, int64_t nseq, 
  * pairs are grouped by the configuration their threshold is tuned to and,
  * inside a group, by length class (ceil(len/32) words); each group runs the
  * tuned mapping (threads per pair, work chunk) in one persistent launch.
- * Batches below pf_set_small_batch's size take one plain launch (with one
- * threshold for the batch, E NULL and E_max <= 15, the plain kernel with
- * that threshold fixed at compile time).
+ * Batches below pf_set_small_batch's size take one launch: the plain kernel
+ * (with one threshold for the batch, E NULL and E_max <= 15, fixed at
+ * compile time), one warp per pair, or, after grouping the pairs by
+ * threshold, a bit-sliced kernel, by size and E_max.
  *   deciders  PF_SNEAKYSNAKE, PF_GATEKEEPER or both (two output slots)
  *   lens      device int32[n], pair lengths
  *   E         device int16[n] per-pair thresholds, or NULL for E_max for
@@ -248,9 +249,9 @@ PF_API pf_status pf_tune_batch(pf_ctx *ctx, unsigned deciders, const pf_pairs *p
                                const int32_t *lens, const int16_t *E, int E_max, int64_t n,
                                int64_t sample, int reps);
 
-/* Batches of fewer than `pairs` pairs skip the scheduler: one launch of the
- * plain one-thread-per-pair kernel serving E_max, no binning and no
- * per-threshold launches, whose fixed costs dominate small batches.
+/* Batches of fewer than `pairs` pairs skip the scheduler's per-threshold
+ * launches, whose fixed costs dominate small batches: one launch serves every
+ * threshold (see pf_filter).
  * Default 2^20; 0 sends every batch of pf_filter / pf_filter_verify /
  * pf_run_host through the batched scheduler (unless pf_tune chose the
  * plain kernel).  PF_EINVAL for pairs < 0. */

@@ -101,23 +101,23 @@ bin_hist_kernel(const int16_t *E, const int32_t *lens, int64_t n, int E_max, Bin
         if (cnt[i]) atomicAdd(&hist[i], (unsigned long long)cnt[i]);
 }
 
-// One warp: exclusive scan of the key counts into the scatter's cursors; a
-// configuration's bin starts at its first key.  When every pair falls in
+// One warp: exclusive scan of the key counts of nbins configurations (or
+// thresholds) into the scatter's cursors; a bin starts at its first key.  When every pair falls in
 // one configuration the grouping is the identity: `ident` tells the
 // scatter to skip and the filter to index pairs directly (pair order is
 // kept; the length classes are not separated).
 __global__ void bin_scan_kernel(const unsigned long long *hist, int64_t *bin_start,
-                                unsigned long long *cursor, int *ident) {
-    constexpr int kPer = (kNumBinKeys + 31) / 32;
+                                unsigned long long *cursor, int *ident, int nbins) {
+    const int nkeys = nbins * kLenClasses, per = (nkeys + 31) / 32;
     __shared__ unsigned long long h[kNumBinKeys];
     const int lane = threadIdx.x;
     if (lane >= 32) return;
-    for (int i = lane; i < kNumBinKeys; i += 32) h[i] = hist[i];  // independent loads
+    for (int i = lane; i < nkeys; i += 32) h[i] = hist[i];  // independent loads
     __syncwarp();
     int64_t sum = 0;
-    for (int k = 0; k < kPer; ++k) {
-        const int i = lane * kPer + k;
-        if (i < kNumBinKeys) sum += (int64_t)h[i];
+    for (int k = 0; k < per; ++k) {
+        const int i = lane * per + k;
+        if (i < nkeys) sum += (int64_t)h[i];
     }
     int64_t inc = sum;
 #pragma unroll
@@ -126,19 +126,19 @@ __global__ void bin_scan_kernel(const unsigned long long *hist, int64_t *bin_sta
         if (lane >= o) inc += t;
     }
     int64_t run = inc - sum;
-    for (int k = 0; k < kPer; ++k) {
-        const int i = lane * kPer + k;
-        if (i >= kNumBinKeys) break;
+    for (int k = 0; k < per; ++k) {
+        const int i = lane * per + k;
+        if (i >= nkeys) break;
         cursor[i] = (unsigned long long)run;
         if (i % kLenClasses == 0) bin_start[i / kLenClasses] = run;
         run += (int64_t)h[i];
     }
-    if (lane == 31) bin_start[kNumBatchCfgs] = inc;
+    if (lane == 31) bin_start[nbins] = inc;
     int used = 0;
-    for (int c0 = 0; c0 < kNumBatchCfgs; c0 += 32) {
+    for (int c0 = 0; c0 < nbins; c0 += 32) {
         const int c = c0 + lane;
         bool any = false;
-        if (c < kNumBatchCfgs)
+        if (c < nbins)
             for (int j = 0; j < kLenClasses; ++j) any |= h[c * kLenClasses + j] != 0ull;
         used += __popc(__ballot_sync(0xffffffffu, any));
     }
@@ -186,6 +186,33 @@ bin_scatter_kernel(const int16_t *E, const int32_t *lens, int64_t n, int E_max, 
             if (key[k] >= 0) order[base[key[k]] + rank[k]] = p0 + k * 256;
         __syncthreads();  // cnt and base are reused by the next tile
     }
+}
+
+// Group the pairs: bin t.cfg_of_E[E], E clamped to [0, E_max], of nbins bins.
+static cudaError_t launch_binning(const FilterArgs &a, const BinTable &t, int nbins,
+                                  const Scratch &s, int sms, cudaStream_t st) {
+    bin_init_kernel<<<1, 256, 0, st>>>(s.bin_start, s.work, s.hist, kNumBatchCfgs, -1, a.n);
+    const int64_t hh = std::max<int64_t>(
+        1, std::min<int64_t>((a.n + 256 * kHistPer - 1) / (256 * kHistPer), (int64_t)sms * 8));
+    bin_hist_kernel<<<(unsigned)hh, 256, 0, st>>>(a.E, a.lens, a.n, a.E_max, t, s.hist);
+    bin_scan_kernel<<<1, 32, 0, st>>>(s.hist, s.bin_start, s.cursor, s.ident, nbins);
+    bin_scatter_kernel<<<(unsigned)hh, 256, 0, st>>>(a.E, a.lens, a.n, a.E_max, t, s.cursor,
+                                                     s.order, s.ident);
+    return cudaGetLastError();
+}
+
+// Whether the pairs that a bin runs together lie together: *scattered = 0 when
+// most of 1,024 sampled neighbours in the bins' order are neighbours in the
+// read's planes (the layout grouped by threshold and length), else 1.
+__global__ void __launch_bounds__(1024)
+bin_layout_kernel(SeqView read, const int32_t *lens, const int64_t *order, const int *ident,
+                  int64_t n, int *scattered) {
+    const int64_t q = (int64_t)((double)threadIdx.x / 1024.0 * (double)(n - 1));
+    const bool id = *ident != 0;
+    const int64_t p = id ? q : order[q], p2 = id ? q + 1 : order[q + 1];
+    const bool near = read.start(p2) - read.start(p) == (int64_t)((lens[p] + 31) >> 5);
+    const int c = __syncthreads_count(near);
+    if (threadIdx.x == 0) *scattered = c < 512;
 }
 
 }  // namespace pf
@@ -250,7 +277,7 @@ pf_status pf_ctx::scratch_layout(int64_t n, Scratch *s) {
     const size_t o_work = off;  off += up(kWorkCounters * sizeof(unsigned long long));
     const size_t o_hist = off;  off += up(kNumBinKeys * sizeof(unsigned long long));
     const size_t o_cur = off;   off += up(kNumBinKeys * sizeof(unsigned long long));
-    const size_t o_ident = off; off += up(sizeof(int));
+    const size_t o_ident = off; off += up(2 * sizeof(int));
     const size_t o_need = off;  off += up(nn);
     pf_status st = ensure_scratch(off);
     if (st != PF_OK) return st;
@@ -281,19 +308,19 @@ int pf_ctx::grid_for(int dec, int cfg) {
 }
 
 // Default configuration for threshold E before any tuning.  The bit-sliced
-// kernels from the threshold on at which their fixed cost (transposing the
-// planes) is less than what they save per diagonal.  Measured at 100, 150 and
-// 250 bp (4M, 4M, 2M pairs; ms, best word-per-pair kernel -> bit-sliced):
-// SneakySnake alone E = 5 0.24 -> 0.22, 0.28 -> 0.28, (E = 4) 0.24 -> 0.26; E = 6
-// (150, 250) 0.31 -> 0.29, 0.29 -> 0.26; both deciders E = 5 0.32 -> 0.26,
-// 0.37 -> 0.33, (E = 4) 0.24 -> 0.29, (E = 6) 0.34 -> 0.33; GateKeeper alone, which
-// has no walk to save, E = 8 0.28 -> 0.26, 0.33 -> 0.34, 0.26 -> 0.32, E = 15
-// (150) 0.58 -> 0.46.  Below, the exact-threshold one-thread kernel (its
-// two-phase form for E = 1..7, with shared arrays that hold pairs up to 256
-// bases).
+// kernels from the threshold on at which they win whatever the lengths (in a
+// tile of mixed lengths every pair is walked to the longest one's end; the
+// tuner finds them lower down where lengths agree).  Filter, ms, best
+// word-per-pair kernel -> bit-sliced: 3M pairs of 100/150/250 bp mixed in pair order,
+// one threshold: both deciders E = 6 0.48 -> 0.56, 12 1.60 -> 0.80, SneakySnake
+// alone E = 8 0.66 -> 0.50, GateKeeper alone E = 12 0.54 -> 0.70; 4M pairs of
+// 150 bp: both E = 6 0.44 -> 0.36, 7 0.50 -> 0.36, SneakySnake E = 6 0.31 -> 0.29,
+// 7 0.38 -> 0.30, GateKeeper E = 15 0.58 -> 0.46; 2M of 250 bp: both E = 6
+// 0.34 -> 0.33, GateKeeper E = 8 0.26 -> 0.32, 20 0.83 -> 0.43.  Below, the
+// exact-threshold one-thread kernel (its two-phase form for E = 1..7, with
+// shared arrays that hold pairs up to 256 bases).
 int pf::pf_default_cfg(int dec, int E) {
-    const int sliced_from = dec == 2 ? 12 : (dec == 1 ? 6 : 5);
-    if (E >= sliced_from)
+    if (E >= (dec == 2 ? 16 : 7))
         for (int c = 0; c < kNumBatchCfgs; ++c)
             if (kBatchCfgs[c].xe == E && cfg_sliced(kBatchCfgs[c])) return c;
     if (E >= 1 && E <= 7)
@@ -362,7 +389,7 @@ static FilterArgs make_filter_args(pf_ctx *ctx, const pf_pairs *pairs, const int
 // ---------------------------------------------------------------------------
 // scheduler
 
-pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &s) {
+pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &s, int cfg) {
     BatchArgs b;
     b.f = a;
     b.bin_start = s.bin_start;
@@ -372,8 +399,8 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
     b.chunk_start = nullptr;
     std::vector<int> used;
     int single = -1;
-    if (!a.E) {
-        single = tune_cfg[dec][a.E_max];
+    if (cfg >= 0 || !a.E) {
+        single = cfg >= 0 ? cfg : tune_cfg[dec][a.E_max];
         used.push_back(single);
         b.order = nullptr;
     } else {
@@ -389,20 +416,16 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
     }
     b.ident = (single < 0) ? s.ident : nullptr;
     binned = single < 0;
-    bin_init_kernel<<<1, 32, 0, stream>>>(s.bin_start, s.work, s.hist, kNumBatchCfgs, single,
-                                          a.n);
+    pf_status st = PF_OK;
     if (single < 0) {
         BinTable t;
         for (int e = 0; e <= PF_MAX_E; ++e) t.cfg_of_E[e] = tune_cfg[dec][std::min(e, a.E_max)];
-        const int64_t hh = std::min<int64_t>((a.n + 256 * kHistPer - 1) / (256 * kHistPer),
-                                             (int64_t)sms * 8);
-        bin_hist_kernel<<<(unsigned)std::max<int64_t>(hh, 1), 256, 0, stream>>>(
-            a.E, a.lens, a.n, a.E_max, t, s.hist);
-        bin_scan_kernel<<<1, 32, 0, stream>>>(s.hist, s.bin_start, s.cursor, s.ident);
-        bin_scatter_kernel<<<(unsigned)std::max<int64_t>(hh, 1), 256, 0, stream>>>(
-            a.E, a.lens, a.n, a.E_max, t, s.cursor, s.order, s.ident);
+        st = cuda(launch_binning(a, t, kNumBatchCfgs, s, sms, stream), "binning launch");
+    } else {
+        bin_init_kernel<<<1, 256, 0, stream>>>(s.bin_start, s.work, s.hist, kNumBatchCfgs, single,
+                                               a.n);
+        st = cuda(cudaGetLastError(), "binning launch");
     }
-    pf_status st = cuda(cudaGetLastError(), "binning launch");
     if (st != PF_OK) return st;
 
     if (used.size() == 1) {
@@ -418,21 +441,71 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
                                                 std::max<int64_t>(1, (steps + wpb - 1) / wpb));
         return cuda(launch_filter_batched(dec, c, grid, b, c, stream), "filter launch");
     }
-    // several configurations: one persistent launch each, concurrently
+    // Several configurations: one persistent launch each, concurrently.  Where
+    // that leaves the average bin less than a wave of bit-sliced tiles (12
+    // warps of 256 pairs per SM), the bit-sliced ones share a launch per class.
+    // Pairs scattered over the planes (and batches too short for whole classes)
+    // take the launch with 16 lanes per group instead, whose segments hold four
+    // words of a pair.  Filter with both deciders, ms, launch per threshold /
+    // per class / 16 lanes: thresholds 0..25, grouped layout, 1.1M pairs 0.65 /
+    // 0.43 / 0.37, 3M 0.94 / 0.71 / 0.91; in pair order 3M 2.57 / 2.22 / 1.02; 1.1M
+    // pairs of eight thresholds up to 20, grouped 0.35 / 0.30 / 0.31.
+    SliceBins sliced{};
+    for (int e = 0; e <= a.E_max; ++e) {
+        const int c = tune_cfg[dec][e];
+        if (!cfg_sliced(kBatchCfgs[c])) continue;
+        sliced.bin[sliced.count] = (unsigned char)c;
+        sliced.E[sliced.count++] = (unsigned char)e;
+    }
+    const bool few = a.n < 1600000;
+    if (sliced.count && !few) {
+        bin_layout_kernel<<<1, 1024, 0, stream>>>(a.pairs.read, a.lens, s.order, s.ident, a.n,
+                                                  s.ident + 1);
+        b.layout = s.ident + 1;
+    }
+    const bool merge = a.n / (int64_t)used.size() < (int64_t)sms * 12 * 256;
     cudaEventRecord(ev_fork, stream);
-    for (size_t i = 0; i < used.size(); ++i) {
-        cudaStream_t side = side_streams[i % kSideStreams];
-        cudaStreamWaitEvent(side, ev_fork, 0);
-        const int c = used[i];
+    int next = 0;   // side streams in turn
+    auto side = [&]() {
+        cudaStream_t x = side_streams[next % kSideStreams];
+        if (next++ < kSideStreams) cudaStreamWaitEvent(x, ev_fork, 0);
+        return x;
+    };
+    if (sliced.count) {
+        b.want = 1;
+        st = cuda(launch_filter_slices((int)dec, 16, b, sliced, -1, sms, side()), "filter launch");
+        b.want = 0;
+        if (st != PF_OK) return st;
+    }
+    if (few || merge) {
+        // the larger thresholds first
+        for (int cls = kSliceClasses - 1; cls >= 0; --cls) {
+            SliceBins bins{};
+            for (int i = 0; i < sliced.count; ++i) {
+                const int e = sliced.E[i];
+                if (!few && (e > kSliceClassE[cls] || (cls && e <= kSliceClassE[cls - 1]))) continue;
+                const auto at = std::find(used.begin(), used.end(), (int)sliced.bin[i]);
+                if (at == used.end()) continue;
+                used.erase(at);
+                bins.bin[bins.count] = sliced.bin[i];
+                bins.E[bins.count++] = (unsigned char)e;
+            }
+            if (few || !bins.count) continue;
+            st = cuda(launch_filter_slice_bins((int)dec, cls, b, bins, sms, side()),
+                      "filter launch");
+            if (st != PF_OK) return st;
+        }
+    }
+    for (const int c : used) {
         BatchArgs bi = b;
         bi.chunk = 256;
         for (int e = 0; e <= a.E_max; ++e)
             if (tune_cfg[dec][e] == c) bi.chunk = tune_chunk[dec][e];
         const int grid = grid_for(dec, c);
-        st = cuda(launch_filter_batched(dec, c, grid, bi, c, side), "filter launch");
+        st = cuda(launch_filter_batched(dec, c, grid, bi, c, side()), "filter launch");
         if (st != PF_OK) return st;
     }
-    for (int i = 0; i < kSideStreams && i < (int)used.size(); ++i) {
+    for (int i = 0; i < kSideStreams && i < next; ++i) {
         cudaEventRecord(ev_join[i], side_streams[i]);
         cudaStreamWaitEvent(stream, ev_join[i], 0);
     }
@@ -649,13 +722,76 @@ static int plain_index(int E_max) {
     return pi;
 }
 
+// How a batch below small_batch runs.  Measured (us) on 150 bp and on the mix of
+// 100/150/250 bp with thresholds of 0 to 10 % (E_max = 25), both deciders
+// unless said otherwise:
+//   wide    one warp per pair, the fused loop: the shortest latency.  Mix, plain
+//           -> wide: 1k pairs 65 -> 14, 16k 82 -> 37, 32k 96 -> 56 (bit-sliced 68);
+//           E_max = 15: 1k 27 -> 13, 16k 27 -> 32
+//   sliced  grouped by threshold, then one bit-sliced launch with 16 lanes per
+//           group of 32 pairs (8 from 100k pairs of one threshold on).  Mix, plain ->
+//           sliced: 100k 265 -> 81, 1M 2609 -> 367; E_max = 15: 32k 29 -> 47,
+//           100k 74 -> 57; one threshold, 100k: E = 8 27 -> 29 (SneakySnake
+//           alone 29 -> 23), 10 36 -> 29, 12 46 -> 29, 25 (250 bp) 206 -> 56; 16k
+//           E = 12 21 -> 20; 50k E = 10 27 -> 23.  GateKeeper alone, mix: 100k 68 -> 68,
+//           200k 133 -> 88; up to E_max = 15 plain is as fast
+//   batched the scheduler with one bin: one threshold, 1M pairs, sliced ->
+//           batched: E = 8 173 -> 115, 12 172 -> 144; 400k 78 -> 83
+//   plain   one thread per pair, everything else
+int pf_ctx::small_route(unsigned dec, const FilterArgs &a) const {
+    const bool gk = dec == 2;
+    if (!a.E) {
+        if (a.n >= 450000 && !tune_plain[dec][a.E_max] &&
+            cfg_sliced(kBatchCfgs[pf_default_cfg((int)dec, a.E_max)]))
+            return kSmallBatched;
+        if (a.E_max < (gk ? 16 : 8)) return kSmallPlain;
+        if (a.E_max >= 16 && a.n < 8000) return kSmallWide;
+        const int64_t plain_below = a.E_max >= 16   ? 0
+                                    : a.E_max >= 12 ? 25000
+                                    : a.E_max >= 10 ? 50000
+                                    : dec == 1      ? 75000
+                                                    : 450000;
+        if (a.n < plain_below) return kSmallPlain;
+        return a.n < 100000 ? 16 : 8;
+    }
+    if (a.E_max < (gk ? 16 : 8)) return kSmallPlain;
+    if (a.n <= (a.E_max >= 16 && !gk ? 40000 : 10000)) return kSmallWide;
+    if ((a.E_max < 16 && a.n < 75000) || (gk && a.n < 100000)) return kSmallPlain;
+    return 16;
+}
+
 pf_status pf_ctx::run_filter(unsigned dec, const FilterArgs &a, const Scratch &s) {
-    // small batches: fixed costs of binning and per-bin launches dominate;
+    // small batches: the fixed costs of per-threshold launches dominate;
     // otherwise the plain kernel where pf_tune found it fastest for every
     // threshold the batch can hold
     binned = false;
     bool plain = a.n < small_batch;
-    if (!plain) {
+    if (plain) {
+        const int route = small_route(dec, a);
+        if (route == kSmallBatched) return run_batched(dec, a, s);
+        if (route == kSmallWide) return run_batched(dec, a, s, kWideCfg);
+        if (route > 0) {
+            BatchArgs b{};
+            b.f = a;
+            if (a.E) {
+                BinTable t;
+                for (int e = 0; e <= PF_MAX_E; ++e) t.cfg_of_E[e] = e;
+                const pf_status st = cuda(launch_binning(a, t, PF_MAX_E + 1, s, sms, stream),
+                                          "binning launch");
+                if (st != PF_OK) return st;
+                b.order = s.order;
+                b.ident = s.ident;
+                b.bin_start = s.bin_start;
+                binned = true;
+            }
+            SliceBins bins{};
+            for (int e = 0; e <= a.E_max; ++e) bins.bin[e] = bins.E[e] = (unsigned char)e;
+            bins.count = a.E_max + 1;
+            return cuda(launch_filter_slices((int)dec, route, b, bins, a.E ? -1 : a.E_max, sms,
+                                             stream),
+                        "filter launch");
+        }
+    } else {
         plain = true;
         for (int e = a.E ? 0 : a.E_max; e <= a.E_max && plain; ++e) plain = tune_plain[dec][e];
     }
@@ -820,13 +956,10 @@ pf_status pf_tune_batch(pf_ctx *ctx, unsigned deciders, const pf_pairs *pairs,
     // group the pairs by threshold: bin e holds the pairs with E = e
     BinTable t;
     for (int e = 0; e <= PF_MAX_E; ++e) t.cfg_of_E[e] = e;
-    bin_init_kernel<<<1, 32, 0, ctx->stream>>>(s.bin_start, s.work, s.hist, kNumBatchCfgs, -1, n);
-    const int64_t hh = std::max<int64_t>(
-        1, std::min<int64_t>((n + 256 * kHistPer - 1) / (256 * kHistPer), (int64_t)ctx->sms * 8));
-    bin_hist_kernel<<<(unsigned)hh, 256, 0, ctx->stream>>>(E, lens, n, E_max, t, s.hist);
-    bin_scan_kernel<<<1, 32, 0, ctx->stream>>>(s.hist, s.bin_start, s.cursor, s.ident);
-    bin_scatter_kernel<<<(unsigned)hh, 256, 0, ctx->stream>>>(E, lens, n, E_max, t, s.cursor,
-                                                               s.order, s.ident);
+    const FilterArgs grouped = make_filter_args(ctx, pairs, lens, E, E_max, nullptr, nullptr, n);
+    st = ctx->cuda(launch_binning(grouped, t, PF_MAX_E + 1, s, ctx->sms, ctx->stream),
+                   "pf_tune_batch bins");
+    if (st != PF_OK) return st;
     int64_t starts[PF_MAX_E + 2];
     std::vector<unsigned long long> keys(kNumBinKeys);
     int ident = 0;

@@ -48,8 +48,8 @@ struct pf_ctx {
     int tune_cfg[4][PF_MAX_E + 1];
     bool tune_plain[4][PF_MAX_E + 1] = {};  // pf_tune found the plain kernel fastest
     int tune_chunk[4][PF_MAX_E + 1];
-    // batches of fewer pairs take one plain launch (no binning, no per-bin
-    // launches); 0 sends every batch through the batched scheduler
+    // batches of fewer pairs take one launch (small_route), no per-bin
+    // launches; 0 sends every batch through the batched scheduler
     int64_t small_batch = int64_t(1) << 20;
     bool resolve_bounds = true;  // skip verifying pairs whose count bounds agree
     // what pf_last_verified_count reads: 0 nothing, 1 the count at the start
@@ -72,8 +72,14 @@ struct pf_ctx {
     pf_status scratch_layout(int64_t n, pf::Scratch *s);
     int grid_for(int dec, int cfg);
     void reset_tuning();
-    pf_status run_batched(unsigned dec, const pf::FilterArgs &a, const pf::Scratch &s);
-    // run_batched, or one plain launch for a batch below small_batch
+    // through the scheduler: every threshold by its tuned configuration, or the
+    // whole batch by configuration cfg
+    pf_status run_batched(unsigned dec, const pf::FilterArgs &a, const pf::Scratch &s,
+                          int cfg = -1);
+    // lanes per group of the bit-sliced small-batch kernel, or one of
+    enum { kSmallPlain = 0, kSmallWide = -1, kSmallBatched = -2 };
+    int small_route(unsigned dec, const pf::FilterArgs &a) const;
+    // run_batched, or one launch for a batch below small_batch
     pf_status run_filter(unsigned dec, const pf::FilterArgs &a, const pf::Scratch &s);
 };
 

@@ -20,6 +20,14 @@ cudaError_t launch_sliced_1(int, int, const BatchArgs &, int, cudaStream_t);
 cudaError_t launch_sliced_5(int, int, const BatchArgs &, int, cudaStream_t);
 cudaError_t launch_sliced_6(int, int, const BatchArgs &, int, cudaStream_t);
 cudaError_t launch_sliced_7(int, int, const BatchArgs &, int, cudaStream_t);
+cudaError_t launch_small_1(int, const BatchArgs &, const SliceBins &, int, int, cudaStream_t);
+cudaError_t launch_small_5(int, const BatchArgs &, const SliceBins &, int, int, cudaStream_t);
+cudaError_t launch_small_6(int, const BatchArgs &, const SliceBins &, int, int, cudaStream_t);
+cudaError_t launch_small_7(int, const BatchArgs &, const SliceBins &, int, int, cudaStream_t);
+cudaError_t launch_slice_bins_1(int, const BatchArgs &, const SliceBins &, int, cudaStream_t);
+cudaError_t launch_slice_bins_5(int, const BatchArgs &, const SliceBins &, int, cudaStream_t);
+cudaError_t launch_slice_bins_6(int, const BatchArgs &, const SliceBins &, int, cudaStream_t);
+cudaError_t launch_slice_bins_7(int, const BatchArgs &, const SliceBins &, int, cudaStream_t);
 const void *sliced_ptr_1(int);
 const void *sliced_ptr_6(int);
 const void *sliced_ptr_7(int);
@@ -34,6 +42,30 @@ cudaError_t launch_filter_sliced(int dec, int cfg, int grid, const BatchArgs &b,
                             : launch_sliced_1(cfg, grid, b, bin, st);
         case 2: return launch_sliced_6(cfg, grid, b, bin, st);
         case 3: return launch_sliced_7(cfg, grid, b, bin, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_filter_slice_bins(int dec, int cls, const BatchArgs &b, const SliceBins &bins,
+                                     int sms, cudaStream_t st) {
+    switch (dec) {
+        case 1:
+            return b.f.need ? launch_slice_bins_5(cls, b, bins, sms, st)
+                            : launch_slice_bins_1(cls, b, bins, sms, st);
+        case 2: return launch_slice_bins_6(cls, b, bins, sms, st);
+        case 3: return launch_slice_bins_7(cls, b, bins, sms, st);
+    }
+    return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_filter_slices(int dec, int lanes, const BatchArgs &b, const SliceBins &bins,
+                                 int single, int sms, cudaStream_t st) {
+    switch (dec) {
+        case 1:
+            return b.f.need ? launch_small_5(lanes, b, bins, single, sms, st)
+                            : launch_small_1(lanes, b, bins, single, sms, st);
+        case 2: return launch_small_6(lanes, b, bins, single, sms, st);
+        case 3: return launch_small_7(lanes, b, bins, single, sms, st);
     }
     return cudaErrorInvalidValue;
 }

@@ -107,6 +107,10 @@ struct BatchArgs {
     unsigned long long *work;    // work-item counter (scratch, zeroed)
     const int64_t *chunk_start;  // [nbins+1] first work item of each bin
     const int *ident;            // device flag: order is the identity (one bin used)
+    // non-null: device flag, 1 when the pairs of a bin are scattered over the
+    // planes; a launch does its work only where the flag equals `want`
+    const int *layout = nullptr;
+    int want = 0;
 };
 
 }  // namespace pf

@@ -76,15 +76,39 @@ constexpr bool cfg_sliced(const KernelCfg &c) { return c.sliced; }
 
 // A bit-sliced warp's tile: columns per block of the walk, words per segment
 // and words of shared memory (SliceColumns).
-__host__ __device__ constexpr int slice_block(int L) { return L == 8 ? 8 : 4; }
+__host__ __device__ constexpr int slice_block(int L) { return L >= 8 ? 8 : 4; }
 __host__ __device__ constexpr int slice_seg(int L) { return L / 4; }
 __host__ __device__ constexpr size_t slice_smem_words(int L) {
-    return (size_t)3 * (32 / L) * (32 * (slice_seg(L) + 2) + slice_block(L) - 1 + 32 * slice_seg(L));
+    return (size_t)3 * (32 / L) *
+           (32 * (slice_seg(L) + 2) + slice_block(L) - 1 + 32 * slice_seg(L));
 }
-// Warps per SM that a kernel's registers are held to: 168 each, or 255 where
-// the diagonals of a lane need them (GateKeeper also keeps four columns of
-// each).  At 128 registers (16 warps) the kernels were no faster.
-constexpr int slice_warps(int DPT, bool gatekeeper) { return DPT <= (gatekeeper ? 6 : 8) ? 12 : 8; }
+// and the bytes with the starts of its pairs where the launch needs them (the
+// smaller, the more L1 is left for the loads: 0.36 against 0.39 ms for 4M pairs
+// of 150 bp at E = 6 without the two tables)
+inline size_t slice_smem_bytes(int L, const BatchArgs &b) {
+    const SeqView &r = b.f.pairs.read, &f = b.f.pairs.ref;
+    const bool strided = !b.order && !r.off && !f.off && r.stride < (1 << 24) && f.stride < (1 << 24);
+    const int tables = strided ? 0 : (r.off == f.off && r.stride == f.stride ? 1 : 2);
+    return slice_smem_words(L) * sizeof(uint32_t) + tables * 32 * (32 / L) * sizeof(int64_t);
+}
+// Warps per SM that a kernel's registers are held to.  More warps hide more
+// latency but leave less L1 for the loads (the walk's arrays take 13.6 KB per
+// warp).  SneakySnake, 12 / 9 warps: 0.285 / 0.283 ms for 4M pairs of 150 bp at
+// E = 6, 0.332 / 0.327 at E = 15, 0.382 / 0.366 for 2M of 250 bp at E = 25; with
+// GateKeeper, which keeps four columns of every diagonal: E = 6 12 / 9 warps
+// 0.353 / 0.359, E = 15 9 / 8 warps 0.503 / 0.535, E = 25 9 (spills) / 8 warps
+// 0.666 / 0.564.
+constexpr int slice_warps(int DPT, bool gatekeeper) {
+    return !gatekeeper ? 9 : (DPT <= 6 ? 12 : (DPT <= 9 ? 9 : 8));
+}
+
+// Bins of several thresholds that one launch takes (launch_filter_slice_bins).
+struct SliceBins {
+    int count;
+    unsigned char bin[32], E[32];  // rising E
+};
+constexpr int kSliceClassE[] = {7, 11, 15, 21, 25};  // largest threshold of each class
+constexpr int kSliceClasses = 5;
 
 // The two-phase form applies where SneakySnake runs (deciders 1 and 3);
 // GateKeeper alone runs a two-phase configuration as the fused loop.
@@ -122,6 +146,8 @@ constexpr int kNumBinKeys = kNumBatchCfgs * kLenClasses;
 // then the verifier's.
 constexpr int kWorkCounters = kNumBatchCfgs + 1;
 constexpr int kFirstExactCfg = 20;  // kBatchCfgs[20 + E] serves exactly E
+constexpr int kWideCfg = 19;        // one warp per pair, every threshold
+static_assert(kBatchCfgs[kWideCfg].tpp == 32 && kBatchCfgs[kWideCfg].ecap == PF_MAX_E);
 
 // Plain kernel (one thread per pair): DPT = kPlainDpt[i] serves E <= DPT - 1.
 constexpr int kPlainDpt[] = {1, 2, 4, 8, 16, 32};
@@ -139,6 +165,14 @@ const void *filter_batched_fn(int dec, int cfg);
 cudaError_t launch_filter_sliced(int dec, int cfg, int grid, const BatchArgs &b, int bin,
                                  cudaStream_t st);
 const void *filter_sliced_fn(int dec, int cfg);
+// One persistent launch over several bit-sliced bins (four lanes per group)
+// whose thresholds belong to class cls.
+cudaError_t launch_filter_slice_bins(int dec, int cls, const BatchArgs &b, const SliceBins &bins,
+                                     int sms, cudaStream_t st);
+// The bit-sliced kernel with more lanes per group: every pair at threshold
+// `single` with 16 or (single >= 8) 8 lanes, or (single < 0) the bins with 16.
+cudaError_t launch_filter_slices(int dec, int lanes, const BatchArgs &b, const SliceBins &bins,
+                                 int single, int sms, cudaStream_t st);
 
 cudaError_t launch_pack_ragged(const uint8_t *ascii, const int64_t *byte_off,
                                const int64_t *word_off, int64_t nseq, uint32_t *lo,

@@ -92,7 +92,7 @@ pf_status alloc_slot(Job &J, Slot &s) {
                  o_tiles = add((size_t)compact_tiles((int64_t)C) * 8),
                  o_bins = add((kNumBatchCfgs + 1) * 8), o_work = add(kWorkCounters * 8),
                  o_hist = add(kNumBinKeys * 8), o_cur = add(kNumBinKeys * 8),
-                 o_ident = add(4), o_need = add(C);
+                 o_ident = add(8), o_need = add(C);
     if (cudaMalloc(&s.mem, o) != cudaSuccess) {
         cudaGetLastError();
         return J.ctx->fail(PF_ENOMEM, "pf_run_host: %zu device bytes per slot", o);

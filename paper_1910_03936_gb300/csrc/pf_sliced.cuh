@@ -20,10 +20,12 @@
 // read's in a ring that also holds the word before and the word after (the
 // band reaches E < 32 columns to either side), the reference's beside it.
 // The split over L lanes and the short segments keep a warp's arrays small
-// (12.6 KB), so that 12 warps share an SM: the walk is a chain of dependent
-// operations per column, and the loads have DRAM's latency.
+// (12.6 KB), so that 8 to 12 warps share an SM: the walk is a chain of
+// dependent operations per column, and the loads have DRAM's latency.
 //
-// What bounds it: neither memory nor the integer pipe alone.  At 150 bp, E = 6,
+// What bounds it: neither memory nor the integer pipe alone, but the loads'
+// way through L1 (a word-wide column of pairs 20 bytes apart takes 20 sectors
+// per 32 words, 9 TB/s from L2) next to the walk's latency.  At 150 bp, E = 6,
 // SneakySnake alone, 4M pairs (0.29 ms), a build without the walk takes 0.19 ms,
 // one without the loads 0.22 ms, one without both 0.11 ms.  Loading the words of
 // a pair together (whole pairs resident: 7 warps per SM; two words per
@@ -33,8 +35,8 @@
 // both deciders).
 //
 // Both deciders, ms, word-per-pair kernels -> this one: 4M pairs of 150 bp at
-// E = 6 0.44 -> 0.36, E = 8 0.58 -> 0.39, E = 15 1.50 -> 0.54; 2M pairs of 250 bp
-// at E = 8 0.48 -> 0.34, E = 20 1.75 -> 0.52, E = 25 2.57 -> 0.57.
+// E = 6 0.44 -> 0.35, E = 8 0.58 -> 0.39, E = 15 1.50 -> 0.50; 2M pairs of 250 bp
+// at E = 8 0.48 -> 0.34, E = 20 1.75 -> 0.52, E = 25 2.12 -> 0.56.
 #pragma once
 #include <climits>
 
@@ -175,7 +177,7 @@ struct SlicePairs {
     int m[G];           // length; -1: absent or invalid
     unsigned invalid;   // bit t: present but its arguments are bad
     int mmin, mmax;     // over the tile's valid pairs (0 when there are none)
-    bool simple;        // all 32 * G pairs present and valid, one length in words, one stride
+    bool whole;         // all 32 * G pairs present and valid, of one length in words
 
     __device__ __forceinline__ int64_t pair(const int64_t *order, int64_t pos, int t) const {
         const int64_t s = pos + 32 * t + (threadIdx.x & 31);
@@ -183,8 +185,7 @@ struct SlicePairs {
     }
 
     __device__ __forceinline__ void load(const int32_t *lens, const int16_t *Es, int E_max, int E,
-                                         const PairsView &pv, const int64_t *order, int64_t pos,
-                                         int cnt) {
+                                         const int64_t *order, int64_t pos, int cnt) {
         const int lane = threadIdx.x & 31;
         invalid = 0u;
         int lo = INT_MAX, hi = 0, wlo = INT_MAX, whi = 0;
@@ -212,8 +213,7 @@ struct SlicePairs {
         whi = (mmax + 31) >> 5;
         all = __all_sync(0xffffffffu, all);
         if (mmin > mmax) mmin = mmax;  // no valid pair
-        simple = all && wlo == whi && !order && !pv.read.off && !pv.ref.off &&
-                 pv.read.stride < (1 << 24) && pv.ref.stride < (1 << 24);
+        whole = all && wlo == whi;
     }
 
     // bit of every pair of the group that has a column i
@@ -229,6 +229,11 @@ struct SlicePairs {
     }
 };
 
+// The two sides' words lie at the same offsets.
+__device__ __forceinline__ bool slice_same(const PairsView &pv) {
+    return pv.read.off == pv.ref.off && pv.read.stride == pv.ref.stride;
+}
+
 // The tile's columns in shared memory.  Read word w's columns lie in slot
 // w % RW of the read's ring (rx: low and high code bit, rn: N), and the
 // ring's first U - 1 columns a second time behind its end, so that a block
@@ -239,16 +244,62 @@ struct SliceColumns {
     static constexpr int RC = 32 * RW + U - 1, FC = 32 * SEG;   // columns
     uint2 *rx, *fx;
     uint32_t *rn, *fn;
+    bool even;                  // the tile's pairs lie one stride apart
+    int64_t rbase, fbase;       // even: first word of the tile's first pair,
+    uint32_t rstep, fstep;      // words from a pair to the next
+    int64_t *rstart, *fstart;   // else first words of the pairs, in shared memory
+                                // (launches over a strided layout in pair order have none)
     int W;              // words of the tile's longest pair
     int w0, nr, nf;     // the next segment's words: first of each side, counts
     int r0;
 
-    __device__ __forceinline__ void init(uint32_t *sm, int mmax) {
+    __device__ __forceinline__ void init(uint32_t *sm, const PairsView &pv,
+                                         const SlicePairs<L> &sp, const int64_t *order,
+                                         int64_t pos) {
         rx = reinterpret_cast<uint2 *>(sm);
         fx = rx + RC * G;
         rn = reinterpret_cast<uint32_t *>(fx + FC * G);
         fn = rn + RC * G;
-        W = (mmax + 31) >> 5;
+        W = (sp.mmax + 31) >> 5;
+        // starts are looked up once: a pair's words are loaded in many rounds
+        const int lane = threadIdx.x & 31;
+        const bool same = slice_same(pv);
+        rstart = reinterpret_cast<int64_t *>(sm + slice_smem_words(L));
+        fstart = rstart + (same ? 0 : 32 * G);
+        even = true;
+        place(pv.read, sp, order, pos, rstart, rbase, rstep);
+        if (same) {
+            fbase = rbase;
+            fstep = rstep;
+        } else {
+            place(pv.ref, sp, order, pos, fstart, fbase, fstep);
+        }
+        even = __all_sync(0xffffffffu, even);
+    }
+
+    // Where one side's pairs lie: evenly spaced (the strided layout, and a
+    // ragged one whose neighbours here are neighbours in memory), or a table.
+    __device__ __forceinline__ void place(const SeqView &v, const SlicePairs<L> &sp,
+                                          const int64_t *order, int64_t pos, int64_t *table,
+                                          int64_t &base, uint32_t &step) {
+        if (!order && !v.off && v.stride < (1 << 24)) {
+            base = pos * v.stride;
+            step = (uint32_t)v.stride;
+            return;
+        }
+        const int lane = threadIdx.x & 31;
+        int64_t st[G];
+#pragma unroll
+        for (int t = 0; t < G; ++t) {
+            st[t] = sp.m[t] > 0 ? v.start(sp.pair(order, pos, t)) : 0;
+            table[32 * t + lane] = st[t];
+        }
+        base = __shfl_sync(0xffffffffu, st[0], 0);
+        const int64_t gap = __shfl_sync(0xffffffffu, st[0], 1) - base;
+        even = even && sp.whole && gap >= 0 && gap < (1 << 24);
+        step = (uint32_t)gap;
+#pragma unroll
+        for (int t = 0; t < G; ++t) even = even && st[t] == base + (32 * t + lane) * gap;
     }
 
     // columns of read word w are N: before the read's start, past its end
@@ -281,8 +332,7 @@ struct SliceColumns {
 
     // Load the 32 words of this lane's job of the round from job j0 on.
     __device__ __forceinline__ void issue(const PairsView &pv, const SlicePairs<L> &sp,
-                                          const int64_t *order, int64_t pos, int j0,
-                                          uint32_t (&x)[32]) {
+                                          int j0, uint32_t (&x)[32]) {
         const int lane = threadIdx.x & 31;
         const int g = lane % G;
         int plane, w;
@@ -290,34 +340,33 @@ struct SliceColumns {
         job(min(j0 + lane / G, 3 * (nr + nf) - 1), ref, plane, w);
         const SeqView &v = ref ? pv.ref : pv.read;
         const uint32_t *src = (plane == 0 ? v.lo : (plane == 1 ? v.hi : v.nm)) + w;
-        if (sp.simple) {
-            const uint32_t step = (uint32_t)(v.stride * G * sizeof(uint32_t));
-            const char *s = reinterpret_cast<const char *>(src + (pos + g) * v.stride);
-#pragma unroll
-            for (int l = 0; l < 32; ++l)
-                x[l] = __ldg(reinterpret_cast<const uint32_t *>(s + (uint64_t)step * l));
-            return;
-        }
+        const uint32_t gap = ref ? fstep : rstep;
+        const uint32_t *first = src + (ref ? fbase : rbase) + (uint64_t)gap * g;
+        const int64_t *st = (ref ? fstart : rstart) + g;
         const uint32_t fill = plane == 2 ? 0xffffffffu : 0u;  // past the end: N
-        if (pv.read.off == pv.ref.off && pv.read.stride == pv.ref.stride) {
-            // the owners of the pairs look their starts up
-            int64_t start[G];
+        if (even) {
+            const char *s = reinterpret_cast<const char *>(first);
+            const uint32_t step = gap * (uint32_t)(G * sizeof(uint32_t));
+            if (sp.whole) {
 #pragma unroll
-            for (int t = 0; t < G; ++t)
-                start[t] = sp.m[t] < 0 ? 0 : pv.read.start(sp.pair(order, pos, t));
+                for (int l = 0; l < 32; ++l)
+                    x[l] = __ldg(reinterpret_cast<const uint32_t *>(s + (uint64_t)step * l));
+                return;
+            }
 #pragma unroll
             for (int l = 0; l < 32; ++l) {
-                const int from = (l % L) * G + g;
-                const int64_t st = __shfl_sync(0xffffffffu, start[l / L], from);
-                const int len = __shfl_sync(0xffffffffu, sp.m[l / L], from);
-                x[l] = len > 32 * w ? __ldg(src + st) : fill;
+                const int len = __shfl_sync(0xffffffffu, sp.m[l / L], (l % L) * G + g);
+                const uint32_t *y = reinterpret_cast<const uint32_t *>(s + (uint64_t)step * l);
+                x[l] = len > 32 * w ? __ldg(y) : fill;
             }
+        } else if (sp.whole) {
+#pragma unroll
+            for (int l = 0; l < 32; ++l) x[l] = __ldg(src + st[l * G]);
         } else {
 #pragma unroll
             for (int l = 0; l < 32; ++l) {
                 const int len = __shfl_sync(0xffffffffu, sp.m[l / L], (l % L) * G + g);
-                const int64_t s = pos + l * G + g;
-                x[l] = len > 32 * w ? __ldg(src + v.start(order ? __ldg(order + s) : s)) : fill;
+                x[l] = len > 32 * w ? __ldg(src + st[l * G]) : fill;
             }
         }
     }
@@ -352,15 +401,14 @@ struct SliceColumns {
     }
 
     // The columns of the segment from word w on.
-    __device__ __forceinline__ void load(const PairsView &pv, const SlicePairs<L> &sp,
-                                         const int64_t *order, int64_t pos, int w) {
+    __device__ __forceinline__ void load(const PairsView &pv, const SlicePairs<L> &sp, int w) {
         plan(w);
         __syncwarp();
         for (int k = max(w ? w + 1 : 0, W); k < w + SEG + 1; ++k) vacant(k);
         const int jobs = 3 * (nr + nf);
         for (int j0 = 0; j0 < jobs; j0 += L) {
             uint32_t x[32];
-            issue(pv, sp, order, pos, j0, x);
+            issue(pv, sp, j0, x);
             transpose32(x);
             store(j0, x);
         }
@@ -368,23 +416,30 @@ struct SliceColumns {
     }
 };
 
-// AND over the group's lanes of N columns each, every lane left with N / L of
-// them (the columns are counted, so it does not matter which).
+// AND over the group's lanes of N columns, which are counted (so it does not
+// matter which lane counts which): every lane is left with N / L of them, or,
+// with more lanes than columns, every L / N-th lane with one and the others
+// with 0.
 template <int G, int O, int N>
 __device__ __forceinline__ void slice_and(uint32_t (&f)[N], uint32_t *out) {
     if constexpr (O < G) {
 #pragma unroll
         for (int i = 0; i < N; ++i) out[i] = f[i];
     } else {
-        static_assert(N % 2 == 0, "columns per block not a multiple of the group's lanes");
         const bool up = (threadIdx.x & O) != 0;
-        uint32_t keep[N / 2];
+        if constexpr (N == 1) {
+            uint32_t v[1] = {f[0] & __shfl_xor_sync(0xffffffffu, f[0], O)};
+            slice_and<G, O / 2, 1>(v, out);
+            if (up) out[0] = 0u;
+        } else {
+            uint32_t keep[N / 2];
 #pragma unroll
-        for (int i = 0; i < N / 2; ++i) {
-            const uint32_t send = up ? f[i] : f[N / 2 + i];
-            keep[i] = (up ? f[N / 2 + i] : f[i]) & __shfl_xor_sync(0xffffffffu, send, O);
+            for (int i = 0; i < N / 2; ++i) {
+                const uint32_t send = up ? f[i] : f[N / 2 + i];
+                keep[i] = (up ? f[N / 2 + i] : f[i]) & __shfl_xor_sync(0xffffffffu, send, O);
+            }
+            slice_and<G, O / 2, N / 2>(keep, out);
         }
-        slice_and<G, O / 2, N / 2>(keep, out);
     }
 }
 
@@ -487,9 +542,10 @@ struct SliceWalk {
                     a[u] = lop3<0xE0>(a[u], t, col(u - 2));                   // & (H | t)
                 }
             }
-            uint32_t mine[U / L];
+            constexpr int NC = U > L ? U / L : 1;
+            uint32_t mine[NC];
             slice_and<G, 16, U>(a, mine);
-            gk.template add<0, U / L>(mine);
+            gk.template add<0, NC>(mine);
 #pragma unroll
             for (int j = 0; j < 4; ++j)
 #pragma unroll
@@ -513,17 +569,17 @@ __device__ __forceinline__ void filter_sliced_tile(const FilterArgs &a, const in
     const int lane = threadIdx.x & 31;
     const int q = lane / G, g = lane % G;
     SlicePairs<L> sp;
-    sp.load(a.lens, a.E, a.E_max, E, a.pairs, order, pos, cnt);
+    sp.load(a.lens, a.E, a.E_max, E, order, pos, cnt);
     const int total = sp.mmax + ((D & 2) ? 2 : 0);  // the last amend looks two columns ahead
     const bool one = sp.mmin == sp.mmax;
     SliceColumns<L> c;
-    c.init(sm, sp.mmax);
+    c.init(sm, a.pairs, sp, order, pos);
     SliceWalk<L, DPT, D> w;
     w.clear();
     __syncwarp();
     c.vacant(-1);
     for (int i0 = 0; i0 < total; i0 += 32 * SEG) {
-        c.load(a.pairs, sp, order, pos, i0 >> 5);
+        c.load(a.pairs, sp, i0 >> 5);
         if (i0 == 0) w.init(c, slice_first<L, DPT>(q, E), E);
         const int cols = min(32 * SEG, total - i0);
         for (int f = 0; f < cols; f += U) {
@@ -568,6 +624,7 @@ template <int L, int DPT, int D>
 __global__ void __launch_bounds__(32, slice_warps(DPT, D & 2))
 filter_sliced_kernel(BatchArgs b, int bin, int E) {
     extern __shared__ __align__(16) uint32_t slice_sm[];
+    if (b.layout && *b.layout != b.want) return;
     constexpr int TILE = SliceShape<L, DPT>::TILE;
     const int64_t lo = b.bin_start[bin], hi = b.bin_start[bin + 1];
     const int64_t *order = (b.order && !(b.ident && *b.ident)) ? b.order : nullptr;
@@ -580,6 +637,111 @@ filter_sliced_kernel(BatchArgs b, int bin, int E) {
         if (threadIdx.x == 0) next = atomicAdd(b.work + bin, 1ull);  // known when this one is done
         filter_sliced_tile<L, DPT, D>(b.f, order, s, (int)min((int64_t)TILE, hi - s), E, slice_sm);
         item = next;
+    }
+}
+
+// A tile of several bins: tile t of the bins' tiles, lane i holding bin i's
+// positions [lo, hi) and the tiles of bins 0..i in inc.
+struct SliceBinScan {
+    int64_t lo, hi, tiles, inc, total;
+
+    template <int TILE>
+    __device__ __forceinline__ void scan(const BatchArgs &b, const SliceBins &bins) {
+        const int lane = threadIdx.x & 31;
+        const int bin = lane < bins.count ? bins.bin[lane] : 0;
+        lo = lane < bins.count ? b.bin_start[bin] : 0;
+        hi = lane < bins.count ? b.bin_start[bin + 1] : 0;
+        span<TILE>();
+    }
+    template <int TILE>
+    __device__ __forceinline__ void span() {
+        const int lane = threadIdx.x & 31;
+        tiles = (hi - lo + TILE - 1) / TILE;
+        inc = tiles;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
+        }
+        total = __shfl_sync(0xffffffffu, inc, 31);
+    }
+    template <int TILE>
+    __device__ __forceinline__ int find(int64_t t, int64_t &pos, int &cnt) const {
+        const int i = __popc(__ballot_sync(0xffffffffu, inc <= t));
+        pos = __shfl_sync(0xffffffffu, lo + (t - (inc - tiles)) * TILE, i);
+        cnt = (int)min((int64_t)TILE, __shfl_sync(0xffffffffu, hi, i) - pos);
+        return i;
+    }
+};
+
+// Several bins in one persistent launch: with a launch per threshold, bins
+// shorter than a wave of warps (0.47M pairs) leave much of the GPU idle.  3M
+// pairs in the grouped layout, both deciders: thresholds 0..25 0.94 -> 0.71 ms,
+// eight thresholds up to 20 0.59 -> 0.56 ms.
+template <int DPT, int D>
+__global__ void __launch_bounds__(32, slice_warps(DPT, D & 2))
+filter_sliced_bins_kernel(BatchArgs b, SliceBins bins) {
+    extern __shared__ __align__(16) uint32_t slice_sm[];
+    constexpr int TILE = SliceShape<4, DPT>::TILE;
+    const int lane = threadIdx.x & 31;
+    const int64_t *order = (b.order && !(b.ident && *b.ident)) ? b.order : nullptr;
+    if (b.layout && *b.layout != b.want) return;
+    SliceBinScan sc;
+    sc.scan<TILE>(b, bins);
+    unsigned long long *work = b.work + bins.bin[0];
+    unsigned long long item = 0, next = 0;
+    if (lane == 0) item = atomicAdd(work, 1ull);
+    for (;;) {
+        item = __shfl_sync(0xffffffffu, item, 0);
+        if ((int64_t)item >= sc.total) break;
+        if (lane == 0) next = atomicAdd(work, 1ull);
+        int64_t s;
+        int cnt;
+        // the largest thresholds first: their tiles take longest
+        const int E = bins.E[sc.find<TILE>(sc.total - 1 - (int64_t)item, s, cnt)];
+        filter_sliced_tile<4, DPT, D>(b.f, order, s, cnt, E, slice_sm);
+        item = next;
+    }
+}
+
+// L lanes per group with L > 4: fewer pairs per warp and longer segments (L / 4
+// words).  For batches too small to fill the GPU with tiles of many groups,
+// where a tile's latency and not the rate counts, and for pairs whose words are
+// scattered over the planes: a segment's words of a pair share sectors.
+// One launch over all tiles of the bins, or, with single >= 0, over the whole
+// batch at that threshold.
+template <int L, int D>
+__global__ void __launch_bounds__(32, L == 8 ? 8 : 12)
+filter_sliced_small_kernel(BatchArgs b, SliceBins bins, int single) {
+    extern __shared__ __align__(16) uint32_t slice_sm[];
+    constexpr int TILE = 32 * (32 / L);
+    if (b.layout && *b.layout != b.want) return;
+    SliceBinScan sc;
+    if (single < 0) {
+        sc.scan<TILE>(b, bins);
+    } else {
+        sc.lo = 0;
+        sc.hi = (threadIdx.x & 31) == 0 ? b.f.n : 0;
+        sc.span<TILE>();
+    }
+    const int64_t *order = (b.order && !(b.ident && *b.ident)) ? b.order : nullptr;
+    // the largest thresholds first: their tiles take longest
+    for (int64_t t = sc.total - 1 - (int64_t)blockIdx.x; t >= 0; t -= gridDim.x) {
+        int64_t s;
+        int cnt;
+        const int i = sc.find<TILE>(t, s, cnt);
+        const int E = single < 0 ? bins.E[i] : single;
+        // diagonals per lane: those of the largest threshold of E's class
+        constexpr int H = L / 2;
+        switch (E >> 3) {
+            case 0:  // (eight lanes take single thresholds from 8 on only)
+                if constexpr (L > 8)
+                    filter_sliced_tile<L, (7 + H) / H, D>(b.f, order, s, cnt, E, slice_sm);
+                break;
+            case 1: filter_sliced_tile<L, (15 + H) / H, D>(b.f, order, s, cnt, E, slice_sm); break;
+            case 2: filter_sliced_tile<L, (23 + H) / H, D>(b.f, order, s, cnt, E, slice_sm); break;
+            default: filter_sliced_tile<L, (31 + H) / H, D>(b.f, order, s, cnt, E, slice_sm); break;
+        }
     }
 }
 

@@ -154,3 +154,34 @@ def test_sides_in_different_layouts(pf, ctx):
     a = pf.pack_pairs(ctx, reads, refs, byte_off=P.read_off)
     b = pf.pack_pairs(ctx, reads, refs, byte_off=P.read_off, group_E=E)
     check(pf, ctx, P, pf.Pairs(a.read, b.ref), E, 25)
+
+
+@pytest.mark.parametrize("n,m,E,E_max", [
+    (700, 0, None, 31),        # one warp per pair
+    (9000, 0, None, 12),
+    (45001, 0, None, 31),      # grouped by threshold, 16 lanes per group
+    (76000, 0, None, 15),
+    (2500, 90, 20, 20),        # one threshold: one warp per pair,
+    (30011, 64, 13, 13),       # 16 lanes,
+    (100031, 40, 25, 25),      # 8 lanes,
+    (100031, 33, 9, 9),
+    (450100, 33, 9, 9),        # the scheduler
+])
+def test_small_batch_routes(pf, n, m, E, E_max):
+    """Each way a batch below the small-batch size can run, at the default
+    setting, on both sides of the lines between them."""
+    if m:
+        P = synth.generate(synth.SKEWED, 31 * n + m, n, m=m, E=E, kmax=40)
+    else:
+        P = synth.generate(synth.SERVE, 17 * n, n, kmax=60)
+        P.E = np.minimum(P.E, E_max).astype(np.int16)
+        if E_max > 25:
+            P.E[::97] = np.arange(len(P.E[::97])) % 32
+    ctx = pf.pf_create(0)
+    try:
+        dev = "cuda:0"
+        reads, refs = torch.from_numpy(P.reads).to(dev), torch.from_numpy(P.refs).to(dev)
+        pairs = pf.pack_pairs(ctx, reads, refs, byte_off=P.read_off)
+        check(pf, ctx, P, pairs, None if m else P.E, E_max)
+    finally:
+        pf.pf_destroy(ctx)
