@@ -174,6 +174,9 @@ cudaError_t launch_filter_slice_bins(int dec, int cls, const BatchArgs &b, const
 cudaError_t launch_filter_slices(int dec, int lanes, const BatchArgs &b, const SliceBins &bins,
                                  int single, int sms, cudaStream_t st);
 
+// SneakySnake on sub-matrices (t columns, y replications), one threshold.
+cudaError_t launch_submat_sliced(const FilterArgs &a, int t, int y, int sms, cudaStream_t st);
+
 cudaError_t launch_pack_ragged(const uint8_t *ascii, const int64_t *byte_off,
                                const int64_t *word_off, int64_t nseq, uint32_t *lo,
                                uint32_t *hi, uint32_t *nm, unsigned *err, cudaStream_t st,

@@ -452,10 +452,16 @@ __device__ __forceinline__ void slice_and(uint32_t (&f)[N], uint32_t *out) {
 // diagonal the column is an obstacle of the snake's: counted, and every
 // diagonal starts afresh at the next column (reset).
 // GateKeeper: column c is amended once column c + 2 is built.
-template <int L, int DPT, int D>
+//
+// SneakySnake on sub-matrices (NBY >= 0, §8.5): every diagonal starts afresh at
+// a sub-matrix's first column as well, and a sub-matrix counts at most y
+// obstacles: NBY bits per pair of the replications left (NBY = 0: y >= t, no
+// sub-matrix has more obstacles than columns).
+template <int L, int DPT, int D, int NBY = -1>
 struct SliceWalk {
     using S = SliceShape<L, DPT>;
     static constexpr int G = S::G, U = S::U, NX = DPT - 1 + U;
+    static constexpr bool SUB = NBY >= 0;
     static constexpr int CAP = 32 * SliceColumns<L>::RW;
     static constexpr bool SS = D & 1, GK = D & 2, HM = D & 4;
 
@@ -465,6 +471,8 @@ struct SliceWalk {
     uint32_t alive[DPT], reset;
     uint32_t hist[4][GK ? DPT : 1];    // mismatch cells of the last four columns
     VCount<S::NB> ss, gk, hm;
+    int t, y, tc;                      // sub-matrix columns, replications; column in it
+    uint32_t left[NBY > 0 ? NBY : 1];
 
     __device__ __forceinline__ void clear() {
         ss.clear();
@@ -508,6 +516,14 @@ struct SliceWalk {
             const uint2 fc = fx[u * G];
             const uint32_t fnm = fn[u * G];
             uint32_t any = 0u;
+            if constexpr (SUB) {
+                if (tc == 0) {
+                    reset = 0xffffffffu;
+#pragma unroll
+                    for (int i = 0; i < NBY; ++i) left[i] = (y >> i) & 1 ? 0xffffffffu : 0u;
+                }
+                tc = tc + 1 == t ? 0 : tc + 1;
+            }
 #pragma unroll
             for (int k = 0; k < DPT; ++k) {
                 uint32_t t = lop3<0xBE>(xc[u + k].x, fc.x, xn[u + k]);  // (x ^ f) | n
@@ -525,6 +541,18 @@ struct SliceWalk {
                 for (int o = G; o < 32; o <<= 1) any |= __shfl_xor_sync(0xffffffffu, any, o);
                 reset = GK ? ~any & v[u] : lop3<0x8A>(any, fnm, v[u]);  // (~any | n) & v
                 obs[u] = reset;
+                if constexpr (NBY > 0) {
+                    uint32_t some = 0u;
+#pragma unroll
+                    for (int i = 0; i < NBY; ++i) some |= left[i];
+                    uint32_t take = obs[u] &= some;
+#pragma unroll
+                    for (int i = 0; i < NBY; ++i) {
+                        const uint32_t b = left[i];
+                        left[i] = b ^ take;
+                        take &= ~b;
+                    }
+                }
             }
         }
         if constexpr (SS) ss.template add<0, U>(obs);
@@ -559,28 +587,26 @@ struct SliceWalk {
     }
 };
 
-// One tile: positions [pos, pos + cnt) of a bin whose pairs all have
-// threshold E (others are invalid), with the warp's arrays at sm.
-template <int L, int DPT, int D>
-__device__ __forceinline__ void filter_sliced_tile(const FilterArgs &a, const int64_t *order,
-                                                   int64_t pos, int cnt, int E, uint32_t *sm) {
+// Walk a tile's columns: positions [pos, pos + cnt) of a bin whose pairs all
+// have threshold E (others are invalid), `extra` columns past the last, with
+// the warp's arrays at sm.
+template <int L, int DPT, typename Walk>
+__device__ __forceinline__ void slice_walk(const FilterArgs &a, const SlicePairs<L> &sp,
+                                           const int64_t *order, int64_t pos, int E, int extra,
+                                           uint32_t *sm, Walk &w) {
     using S = SliceShape<L, DPT>;
     constexpr int G = S::G, U = S::U, SEG = S::SEG;
     const int lane = threadIdx.x & 31;
-    const int q = lane / G, g = lane % G;
-    SlicePairs<L> sp;
-    sp.load(a.lens, a.E, a.E_max, E, order, pos, cnt);
-    const int total = sp.mmax + ((D & 2) ? 2 : 0);  // the last amend looks two columns ahead
+    const int total = sp.mmax + extra;
     const bool one = sp.mmin == sp.mmax;
     SliceColumns<L> c;
     c.init(sm, a.pairs, sp, order, pos);
-    SliceWalk<L, DPT, D> w;
     w.clear();
     __syncwarp();
     c.vacant(-1);
     for (int i0 = 0; i0 < total; i0 += 32 * SEG) {
         c.load(a.pairs, sp, i0 >> 5);
-        if (i0 == 0) w.init(c, slice_first<L, DPT>(q, E), E);
+        if (i0 == 0) w.init(c, slice_first<L, DPT>(lane / G, E), E);
         const int cols = min(32 * SEG, total - i0);
         for (int f = 0; f < cols; f += U) {
             uint32_t v[U];
@@ -596,6 +622,20 @@ __device__ __forceinline__ void filter_sliced_tile(const FilterArgs &a, const in
             w.block(c, f, v);
         }
     }
+}
+
+template <int L, int DPT, int D>
+__device__ __forceinline__ void filter_sliced_tile(const FilterArgs &a, const int64_t *order,
+                                                   int64_t pos, int cnt, int E, uint32_t *sm) {
+    using S = SliceShape<L, DPT>;
+    constexpr int G = S::G;
+    const int lane = threadIdx.x & 31;
+    const int q = lane / G, g = lane % G;
+    SlicePairs<L> sp;
+    sp.load(a.lens, a.E, a.E_max, E, order, pos, cnt);
+    SliceWalk<L, DPT, D> w;
+    // the last amend looks two columns ahead
+    slice_walk<L, DPT>(a, sp, order, pos, E, (D & 2) ? 2 : 0, sm, w);
     if constexpr (D & 2) {
 #pragma unroll
         for (int x = G; x < 32; x <<= 1) w.gk.add_lane(x);
@@ -616,6 +656,34 @@ __device__ __forceinline__ void filter_sliced_tile(const FilterArgs &a, const in
         int gkc = 0;
         if constexpr (D & 2) gkc = h <= E ? h : w.gk.get(l, top);
         write_outputs<D & 3>(a, p, E, ssc, gkc, h);
+    }
+}
+
+// SneakySnake on sub-matrices of t columns with y replications, the whole batch
+// at threshold a.E_max.
+template <int L, int DPT, int NBY>
+__global__ void __launch_bounds__(32, slice_warps(DPT, false))
+submat_sliced_kernel(FilterArgs a, int t, int y) {
+    extern __shared__ __align__(16) uint32_t slice_sm[];
+    using S = SliceShape<L, DPT>;
+    const int lane = threadIdx.x & 31;
+    const int E = a.E_max;
+    for (int64_t pos = (int64_t)blockIdx.x * S::TILE; pos < a.n; pos += (int64_t)gridDim.x * S::TILE) {
+        const int cnt = (int)min((int64_t)S::TILE, a.n - pos);
+        SlicePairs<L> sp;
+        sp.load(a.lens, nullptr, E, E, nullptr, pos, cnt);
+        SliceWalk<L, DPT, 1, NBY> w;
+        w.t = t;
+        w.y = y;
+        w.tc = 0;
+        slice_walk<L, DPT>(a, sp, nullptr, pos, E, 0, slice_sm, w);
+#pragma unroll
+        for (int k = 0; k < S::G; ++k) {
+            if (32 * k + lane >= cnt) continue;
+            const int64_t p = pos + 32 * k + lane;
+            if ((sp.invalid >> k) & 1u) write_invalid<1>(a, p);
+            else write_outputs<1>(a, p, E, w.ss.get(k * L + lane / S::G, E + 1), 0, 0);
+        }
     }
 }
 

@@ -431,6 +431,18 @@ static VariantArgs variant_args_of(pf_ctx *ctx, const pf_pairs *pairs, const int
     return a;
 }
 
+static FilterArgs filter_args_of(const VariantArgs &v) {
+    FilterArgs a;
+    a.pairs = v.pairs;
+    a.lens = v.lens;
+    a.E_max = v.E_max;
+    a.accept = v.accept;
+    a.count = v.count;
+    a.n = v.n;
+    a.err = v.err;
+    return a;
+}
+
 extern "C" pf_status pf_filter_partitioned(pf_ctx *ctx, const pf_pairs *pairs,
                                            const int32_t *lens, const int16_t *E, int E_max,
                                            int t, int y, uint8_t *accept, int16_t *count,
@@ -442,6 +454,17 @@ extern "C" pf_status pf_filter_partitioned(pf_ctx *ctx, const pf_pairs *pairs,
     if (n == 0) return PF_OK;
     cudaSetDevice(ctx->device);
     const VariantArgs a = variant_args_of(ctx, pairs, lens, E, E_max, t, y, accept, count, n);
+    // One threshold: bit-sliced tiles, whose time does not depend on t and y.
+    // One pair per lane group costs about (E + 2) * steps, steps = 32 y / t per
+    // word.  2M pairs of 150 bp, E = 6, t = 8, y = 2 (64): 395 us so, 183 in
+    // tiles; t = 32, y = 1 (8): 177 and 182; 250 bp, E = 25, t = 8, y = 2:
+    // 2810 and 441.  Few pairs leave tiles without enough warps: 100,000 of the
+    // first take 27 us so and 35 in tiles; 1000 of 250 bp, E = 12, t = 8, y = 2
+    // (112) 38 and 28, 30,000 of 150 bp, E = 12, t = 32, y = 4 (56) 19 and 20.
+    const int cost = (E_max + 2) * (32 * std::min(y, t) / t);
+    if (!E && (n >= 150000 ? E_max >= 8 || cost >= 18 : E_max >= 8 && cost >= 56))
+        return ctx->cuda(launch_submat_sliced(filter_args_of(a), t, y, ctx->sms, ctx->stream),
+                         "pf_filter_partitioned launch");
     return ctx->cuda(launch_variant<PartitionedK>(a, ctx->sms, ctx->stream),
                      "pf_filter_partitioned launch");
 }

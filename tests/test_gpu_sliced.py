@@ -185,3 +185,46 @@ def test_small_batch_routes(pf, n, m, E, E_max):
         check(pf, ctx, P, pairs, None if m else P.E, E_max)
     finally:
         pf.pf_destroy(ctx)
+
+
+@pytest.mark.parametrize("t,y", [(8, 2), (8, 8), (5, 3), (32, 32), (1, 1), (13, 4), (32, 1), (32, 31)])
+@pytest.mark.parametrize("n", [300, 200003])
+def test_submatrices_at_one_threshold(pf, t, y, n):
+    """Both forms of the bit-sliced sub-matrix kernel (16 and 4 lanes per
+    group) and what small thresholds take beside them, each count of replication
+    bits, every class of thresholds, lengths mixed in a tile."""
+    dev = "cuda:0"
+    few = n > 1000
+    for E in (0, 4, 7, 11, 15, 20, 25, 31) if not few else (0, 2, 5, 6, 9, 13, 20, 28):
+        rng = np.random.default_rng(E * 100 + t)
+        m = 3000 if few else n
+        lens = rng.choice([0, 1, 31, 33, 64, 65, 100, 127, 150, 161], size=m)
+        P = ragged(E + t, lens, np.full(m, E))
+        ctx = pf.pf_create(0)
+        try:
+            reads, refs = torch.from_numpy(P.reads).to(dev), torch.from_numpy(P.refs).to(dev)
+            pairs = pf.pack_pairs(ctx, reads, refs, byte_off=P.read_off)
+            want = oracle.int_batch("ss_partitioned", P, p0=t, p1=y).copy()
+            if few:   # the same pairs over and over
+                rep = np.arange(n) % m
+                off = pairs.read.word_off[torch.from_numpy(rep).to(dev)].contiguous()
+                pairs.read.word_off = pairs.ref.word_off = off
+                lens, want = P.lens[rep], want[rep]
+            ld = torch.from_numpy(np.ascontiguousarray(lens, dtype=np.int32)).to(dev)
+            acc = torch.full((n,), 9, dtype=torch.uint8, device=dev)
+            cnt = torch.full((n,), 99, dtype=torch.int16, device=dev)
+            pf.pf_filter_partitioned(ctx, pairs, ld, None, E, t, y, acc, cnt, n)
+            pf.pf_sync(ctx)
+            c = cnt.cpu().numpy()
+            assert np.array_equal(c, want), (E, np.nonzero(c != want)[0][:5])
+            assert np.array_equal(acc.cpu().numpy(), (want <= E).astype(np.uint8))
+            if not few:   # a negative length is refused, its neighbours are not
+                ld[5] = -1
+                pf.pf_filter_partitioned(ctx, pairs, ld, None, E, t, y, acc, cnt, n)
+                with pytest.raises(pf.PFError):
+                    pf.pf_sync(ctx)
+                c = cnt.cpu().numpy()
+                assert c[5] == -1 and acc[5].item() == 0
+                assert np.array_equal(np.delete(c, 5), np.delete(want, 5))
+        finally:
+            pf.pf_destroy(ctx)
