@@ -569,6 +569,7 @@ pf_status pf_destroy(pf_ctx *ctx) {
     if (!ctx) return PF_EINVAL;
     cudaSetDevice(ctx->device);
     pf_serve_teardown(ctx);
+    pf_host_teardown(ctx);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     if (ctx->scratch) cudaFree(ctx->scratch);
     if (ctx->d_err) cudaFree(ctx->d_err);

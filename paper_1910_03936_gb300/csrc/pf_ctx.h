@@ -26,6 +26,13 @@ constexpr int kSideStreams = 4;
 
 int pf_default_cfg(int dec, int E);
 
+// What pf_run_host keeps between calls for one of its two slots.
+struct HostSlot {
+    char *mem = nullptr;
+    size_t bytes = 0;
+    cudaStream_t st = nullptr;
+};
+
 }  // namespace pf
 
 struct pf_ctx {
@@ -64,6 +71,8 @@ struct pf_ctx {
     cudaEvent_t ev_fork = nullptr;
     cudaEvent_t ev_join[pf::kSideStreams] = {};
 
+    pf::HostSlot host_slots[2];
+
     pf::ServeState *serve = nullptr;
 
     pf_status fail(pf_status s, const char *fmt, ...);
@@ -84,3 +93,4 @@ struct pf_ctx {
 };
 
 void pf_serve_teardown(pf_ctx *ctx);
+void pf_host_teardown(pf_ctx *ctx);

@@ -1,13 +1,20 @@
 // a7: the whole path on host buffers, in chunks, replayed as CUDA graphs.
 // Contract: pf_run_host in pf.h.
 //
-// Two slots alternate.  A slot owns device buffers for one chunk (ASCII,
-// offsets, planes, outputs, scheduler scratch) and a stream.  Its device
-// work for a chunk -- offsets and lengths, pack of reads and references,
-// the batched filter, compaction, the fill of rejected distances and the
-// verification -- is captured once per chunk size as a CUDA graph and then
-// launched for every chunk, so a chunk costs one graph launch plus its
-// copies.  Chunk c uploads on slot c % 2 while chunk c-1 runs on the other.
+// Two slots alternate.  A slot has device buffers for one chunk (ASCII,
+// offsets, planes, outputs, scheduler scratch) and a stream.  Chunk c uploads
+// on slot c % 2 while chunk c-1 runs on the other.  The device work of a chunk
+// -- offsets and lengths, pack of reads and references, the batched filter,
+// compaction, the fill of rejected distances and the verification -- hides
+// behind the next chunk's upload, so calls of a few chunks enqueue it as it is;
+// with more, full chunks replay a graph captured once per slot.
+//
+// The call is bound by the upload; what it adds is what comes before the first
+// copy and after the last.  So a slot is set up only when its first chunk comes
+// (the second under the first's upload), and its memory and stream stay with
+// the context.  1.5M pairs of 150 bp in two chunks: 3320 us with four graphs
+// captured and both slots allocated and freed by every call, 2380 us now (the
+// upload of 450 MB 2130).
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -42,9 +49,7 @@ __global__ void fill_lens_kernel(int32_t *lens, int64_t n, int len) {
 inline size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct Slot {
-    cudaStream_t st = nullptr;
-    cudaEvent_t ev_done = nullptr;
-    char *mem = nullptr;
+    cudaStream_t st = nullptr;   // the context's, like the memory behind the pointers
     uint8_t *reads = nullptr, *refs = nullptr;
     int64_t *boff_abs = nullptr, *boff = nullptr, *woff = nullptr;
     int32_t *lens = nullptr;
@@ -54,9 +59,16 @@ struct Slot {
     int16_t *cnt = nullptr;
     int32_t *dist = nullptr;
     Scratch scr{};
-    cudaGraphExec_t exec_full = nullptr, exec_tail = nullptr;
-    int64_t c0 = -1, nc = 0;   // chunk in flight
+    cudaGraphExec_t exec = nullptr;   // full chunks
+    int64_t c0 = -1, nc = 0;          // chunk in flight
 };
+
+// Full chunks per call from which on they replay a graph: capturing one per
+// slot costs as much host time as enqueueing a handful of chunks.
+constexpr int64_t kGraphChunks = 8;
+// A slot's memory above this goes back at the end of the call (chunks of 2^20
+// pairs of 250 bp take 0.8 GB).
+constexpr size_t kKeepBytes = size_t(1) << 30;
 
 struct Job {
     pf_ctx *ctx;
@@ -74,7 +86,14 @@ struct Job {
     size_t bytes_max, words_max;
 };
 
-pf_status alloc_slot(Job &J, Slot &s) {
+void release(HostSlot &h) {
+    if (h.mem) cudaFree(h.mem);
+    h.mem = nullptr;
+    h.bytes = 0;
+}
+
+pf_status setup_slot(Job &J, Slot &s, int which) {
+    HostSlot &h = J.ctx->host_slots[which];
     const size_t C = (size_t)J.C, sl = (size_t)J.slots;
     size_t o = 0;
     auto add = [&](size_t b) {
@@ -93,11 +112,22 @@ pf_status alloc_slot(Job &J, Slot &s) {
                  o_bins = add((kNumBatchCfgs + 1) * 8), o_work = add(kWorkCounters * 8),
                  o_hist = add(kNumBinKeys * 8), o_cur = add(kNumBinKeys * 8),
                  o_ident = add(8), o_need = add(C);
-    if (cudaMalloc(&s.mem, o) != cudaSuccess) {
-        cudaGetLastError();
-        return J.ctx->fail(PF_ENOMEM, "pf_run_host: %zu device bytes per slot", o);
+    if (h.bytes < o) {
+        release(h);
+        if (cudaMalloc(&h.mem, o) != cudaSuccess) {
+            cudaGetLastError();
+            h.mem = nullptr;
+            return J.ctx->fail(PF_ENOMEM, "pf_run_host: %zu device bytes per slot", o);
+        }
+        h.bytes = o;
     }
-    char *m = s.mem;
+    if (!h.st && cudaStreamCreateWithFlags(&h.st, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaGetLastError();
+        h.st = nullptr;
+        return J.ctx->fail(PF_ECUDA, "pf_run_host: stream creation failed");
+    }
+    s.st = h.st;
+    char *m = h.mem;
     s.reads = reinterpret_cast<uint8_t *>(m + o_r);
     s.refs = reinterpret_cast<uint8_t *>(m + o_f);
     s.boff_abs = reinterpret_cast<int64_t *>(m + o_ba);
@@ -119,11 +149,6 @@ pf_status alloc_slot(Job &J, Slot &s) {
     s.scr.cursor = reinterpret_cast<unsigned long long *>(m + o_cur);
     s.scr.ident = reinterpret_cast<int *>(m + o_ident);
     s.scr.need = reinterpret_cast<uint8_t *>(m + o_need);
-    if (cudaStreamCreateWithFlags(&s.st, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&s.ev_done, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        return J.ctx->fail(PF_ECUDA, "pf_run_host: stream/event creation failed");
-    }
     if (!J.byte_off) {
         fill_lens_kernel<<<std::max<int64_t>(1, std::min<int64_t>((J.C + 255) / 256, 1024)), 256,
                            0, s.st>>>(s.lens, J.C, J.len);
@@ -187,6 +212,8 @@ pf_status enqueue_chunk(Job &J, Slot &s, int64_t nc) {
 }
 
 pf_status capture(Job &J, Slot &s, int64_t nc, cudaGraphExec_t *exec) {
+    // occupancy queries before the capture
+    for (int c = 0; c < kNumBatchCfgs; ++c) J.ctx->grid_for((int)J.dec, c);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(s.st, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return J.ctx->cuda(e, "pf_run_host capture");
@@ -200,15 +227,6 @@ pf_status capture(Job &J, Slot &s, int64_t nc, cudaGraphExec_t *exec) {
     e = cudaGraphInstantiate(exec, g, 0);
     cudaGraphDestroy(g);
     return J.ctx->cuda(e, "pf_run_host instantiate");
-}
-
-void free_slot(Slot &s) {
-    if (s.st) cudaStreamSynchronize(s.st);
-    if (s.exec_full) cudaGraphExecDestroy(s.exec_full);
-    if (s.exec_tail) cudaGraphExecDestroy(s.exec_tail);
-    if (s.mem) cudaFree(s.mem);
-    if (s.ev_done) cudaEventDestroy(s.ev_done);
-    if (s.st) cudaStreamDestroy(s.st);
 }
 
 // Results of the chunk on slot s into the caller's buffers.
@@ -227,6 +245,14 @@ void copy_out(Job &J, Slot &s) {
 }  // namespace pf
 
 using namespace pf;
+
+void pf_host_teardown(pf_ctx *ctx) {
+    for (HostSlot &h : ctx->host_slots) {
+        release(h);
+        if (h.st) cudaStreamDestroy(h.st);
+        h.st = nullptr;
+    }
+}
 
 extern "C" pf_status pf_run_host(pf_ctx *ctx, unsigned deciders, const uint8_t *reads,
                                  const uint8_t *refs, const int64_t *byte_off, int len,
@@ -258,19 +284,15 @@ extern "C" pf_status pf_run_host(pf_ctx *ctx, unsigned deciders, const uint8_t *
         J.bytes_max = (size_t)J.C * (size_t)len;
         J.words_max = (size_t)J.C * (size_t)((len + 31) / 32);
     }
-    // occupancy queries before any capture
-    for (int c = 0; c < kNumBatchCfgs; ++c) ctx->grid_for((int)deciders, c);
-
     Slot slots[2];
     pf_status st = PF_OK;
-    const int64_t tail = n - (nchunks - 1) * J.C;
-    for (int i = 0; i < 2 && st == PF_OK; ++i) {
-        st = alloc_slot(J, slots[i]);
-        if (st == PF_OK) st = capture(J, slots[i], J.C, &slots[i].exec_full);
-        if (st == PF_OK && tail != J.C) st = capture(J, slots[i], tail, &slots[i].exec_tail);
-    }
+    const bool replay = n / J.C >= kGraphChunks;
     for (int64_t c = 0; c < nchunks && st == PF_OK; ++c) {
         Slot &s = slots[c & 1];
+        if (!s.st) {
+            st = setup_slot(J, s, (int)(c & 1));
+            if (st != PF_OK) break;
+        }
         const int64_t c0 = c * J.C, nc = std::min(J.C, n - c0);
         // the slot's previous chunk: results are in host memory once its
         // copies (queued on the same stream) are done
@@ -286,13 +308,22 @@ extern "C" pf_status pf_run_host(pf_ctx *ctx, unsigned deciders, const uint8_t *
             cudaMemcpyAsync(s.boff_abs, byte_off + c0, (size_t)(nc + 1) * 8, cudaMemcpyHostToDevice,
                             s.st);
         if (E) cudaMemcpyAsync(s.E, E + c0, (size_t)nc * 2, cudaMemcpyHostToDevice, s.st);
-        st = ctx->cuda(cudaGraphLaunch(nc == J.C ? s.exec_full : s.exec_tail, s.st),
-                       "pf_run_host graph launch");
+        if (replay && nc == J.C) {
+            if (!s.exec) st = capture(J, s, nc, &s.exec);
+            if (st == PF_OK)
+                st = ctx->cuda(cudaGraphLaunch(s.exec, s.st), "pf_run_host graph launch");
+        } else {
+            st = enqueue_chunk(J, s, nc);
+        }
         if (st != PF_OK) break;
         copy_out(J, s);
-        cudaEventRecord(s.ev_done, s.st);
     }
-    for (auto &s : slots) free_slot(s);
+    for (auto &s : slots)
+        if (s.st) cudaStreamSynchronize(s.st);
+    for (int i = 0; i < 2; ++i) {
+        if (slots[i].exec) cudaGraphExecDestroy(slots[i].exec);
+        if (ctx->host_slots[i].bytes > kKeepBytes) release(ctx->host_slots[i]);
+    }
     if (st != PF_OK) return st;
     st = ctx->cuda(cudaGetLastError(), "pf_run_host");
     if (st != PF_OK) return st;
