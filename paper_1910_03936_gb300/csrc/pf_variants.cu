@@ -167,32 +167,115 @@ __global__ void __launch_bounds__(256) partitioned_kernel(VariantArgs a) {
 // then updated column by column: the state is its bits c, c+1, c+2 (bit
 // c+3 is still the initial 1, no earlier window reached it); the window's
 // vector replaces the four bits when it has fewer ones, and bit c is final.
+//
+// The kernel is bound by the integer pipe.  A column of the update looks its
+// window's vector up in a table of 16 words (one bank each: lanes never
+// conflict) that hold what each of the eight states becomes, so that the serial
+// chain is a rotation and a mask: 2M pairs of 150 bp, E = 6, 535 us with the
+// vectors put together and their ones counted column by column, 353 so (412 with
+// rows at shifts by d = k - E, a branch and an extra shift each).
 __device__ __forceinline__ uint32_t sel(uint32_t mask, uint32_t a, uint32_t b) {
     return (a & mask) | (b & ~mask);
 }
 
+__device__ __forceinline__ uint32_t majority(uint32_t a, uint32_t b, uint32_t c) {
+    return (a & b) | (c & (a | b));
+}
+
+// The table's word of window vector v.  State s has its field from bit 4 s + 2
+// on (modulo 32): the next state, then the final bit; rotated right by 4 s, the
+// next state's rotation is bits 2..4 and the final bit is bit 5.
+__device__ __forceinline__ uint32_t shouji_steps(unsigned v) {
+    uint32_t t = 0u;
+    for (unsigned s = 0; s < 8; ++s) {
+        const unsigned cur = s | 8u;
+        const unsigned nxt = (__popc(v) < __popc(cur)) ? v : cur;
+        const uint32_t field = (nxt >> 1) | ((nxt & 1u) << 3);
+        t |= __funnelshift_l(field, field, 4 * s + 2);
+    }
+    return t;
+}
+
+// Columns 4 k + J of the planes as nibble k of a word.
+template <int J>
+__device__ __forceinline__ uint32_t nibbles(uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3) {
+    // plane q's bit 4 k + J to bit 4 k + q
+    auto to = [](uint32_t x, int up) { return up >= 0 ? x << up : x >> -up; };
+    return sel(0x33333333u, sel(0x11111111u, to(v0, -J), to(v1, 1 - J)),
+               sel(0x44444444u, to(v2, 2 - J), to(v3, 3 - J)));
+}
+
+// As Cursor, with the read's planes shifted by E once per word: row k = d + E is
+// a shift by a constant, whatever E is.
+template <int EMAX>
+struct BandCursor {
+    int W, w, E;
+    int64_t rb, fb;
+    Word3 S[EMAX > 15 ? 3 : 2];   // read bits from 32 w - E on
+    Word3 last, F;                // the newest read word; the reference's
+    static __device__ __forceinline__ Word3 shift(const Word3 &x, const Word3 &y, int E) {
+        const unsigned s = 32u - (unsigned)E;
+        return {__funnelshift_rc(x.lo, y.lo, s), __funnelshift_rc(x.hi, y.hi, s),
+                __funnelshift_rc(x.nm, y.nm, s)};
+    }
+    static constexpr int N = EMAX > 15 ? 3 : 2;
+    __device__ __forceinline__ void start(const PairsView &pv, int64_t p, int m, int E_) {
+        W = (m + 31) >> 5;
+        w = 0;
+        E = E_;
+        rb = pv.read.start(p);
+        fb = pv.ref.start(p);
+        last = load_word(pv.read, rb, -1, W);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+            const Word3 y = load_word(pv.read, rb, i, W);
+            S[i] = shift(last, y, E);
+            last = y;
+        }
+        F = load_word(pv.ref, fb, 0, W);
+    }
+    __device__ __forceinline__ void next(const PairsView &pv) {
+        ++w;
+        const Word3 y = load_word(pv.read, rb, w + N - 1, W);
+#pragma unroll
+        for (int i = 0; i + 1 < N; ++i) S[i] = S[i + 1];
+        S[N - 1] = shift(last, y, E);
+        last = y;
+        F = load_word(pv.ref, fb, w, W);
+    }
+    __device__ __forceinline__ uint32_t row(int k) const {
+        const Word3 &x = S[k >> 5], &y = S[(k >> 5) + 1];
+        const unsigned o = (unsigned)k & 31u;
+        return (F.lo ^ __funnelshift_r(x.lo, y.lo, o)) | (F.hi ^ __funnelshift_r(x.hi, y.hi, o)) |
+               F.nm | __funnelshift_r(x.nm, y.nm, o);
+    }
+};
+
 template <int EMAX>
 __global__ void __launch_bounds__(256) shouji_kernel(VariantArgs a) {
     constexpr int NSMAX = 2 * EMAX + 1;
+    __shared__ uint32_t steps[16];
+    if (threadIdx.x < 16) steps[threadIdx.x] = shouji_steps(threadIdx.x);
+    __syncthreads();
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.n;
          p += (int64_t)gridDim.x * blockDim.x) {
         int m, E;
         if (!variant_args(a, p, &m, &E)) continue;
         const int ns = 2 * E + 1;
-        Cursor x;
-        x.start(a.pairs, p, m);
+        BandCursor<EMAX> x;
+        x.start(a.pairs, p, m, E);
         uint32_t A[NSMAX], B[NSMAX];
 #pragma unroll
         for (int k = 0; k < NSMAX; ++k)
-            if (k < ns) A[k] = x.map(k - E);
+            if (k < ns) A[k] = x.row(k);
         x.next(a.pairs);
 #pragma unroll
         for (int k = 0; k < NSMAX; ++k)
-            if (k < ns) B[k] = x.map(k - E);
-        unsigned state = 7u;  // bits c, c+1, c+2 of the bit-vector
+            if (k < ns) B[k] = x.row(k);
+        unsigned state = 28u;  // 4 times bits c, c+1, c+2 of the bit-vector
         int ones = 0;
         for (int w = 0; w < x.W && ones <= E; ++w) {
-            uint32_t V0 = 0, V1 = 0, V2 = 0, V3 = 0, K0 = 0, K1 = 0, K2 = 0, K3 = 0;
+            uint32_t V0 = 0, V1 = 0, V2 = 0, V3 = 0, K1 = 0, K2 = 0, K3 = 0;
 #pragma unroll
             for (int k = 0; k < NSMAX; ++k) {
                 if (k >= ns) continue;
@@ -205,38 +288,46 @@ __global__ void __launch_bounds__(256) shouji_kernel(VariantArgs a) {
                 const uint32_t cc = s01 & s23;
                 const uint32_t o0 = s01 ^ s23;
                 const uint32_t o1 = c01 ^ c23 ^ cc;
-                const uint32_t o2 = (c01 & c23) | ((c01 ^ c23) & cc);
-                // cost bits k3 k2 k1 k0 = o2 o1 o0 b0
+                const uint32_t o2 = c01 & c23;
+                // cost bits o2 o1 o0 b0; the best so far K3 K2 K1 V0
                 if (k == 0) {
                     V0 = b0; V1 = b1; V2 = b2; V3 = b3;
-                    K0 = b0; K1 = o0; K2 = o1; K3 = o2;
+                    K1 = o0; K2 = o1; K3 = o2;
                 } else {
-                    // cost < K, per column, most significant bit first
-                    const uint32_t eq3 = ~(o2 ^ K3), eq2 = ~(o1 ^ K2), eq1 = ~(o0 ^ K1);
-                    const uint32_t lt = (~o2 & K3) |
-                                        (eq3 & ((~o1 & K2) | (eq2 & ((~o0 & K1) |
-                                                                      (eq1 & ~b0 & K0)))));
+                    // cost < best, per column: the borrow of their difference
+                    const uint32_t lt =
+                        majority(~o2, K3, majority(~o1, K2, majority(~o0, K1, ~b0 & V0)));
                     V0 = sel(lt, b0, V0); V1 = sel(lt, b1, V1);
                     V2 = sel(lt, b2, V2); V3 = sel(lt, b3, V3);
-                    K0 = sel(lt, b0, K0); K1 = sel(lt, o0, K1);
+                    K1 = sel(lt, o0, K1);
                     K2 = sel(lt, o1, K2); K3 = sel(lt, o2, K3);
                 }
             }
             const int ncol = min(32, m - 32 * w);
-            for (int c = 0; c < ncol; ++c) {
-                const unsigned v = ((V0 >> c) & 1u) | (((V1 >> c) & 1u) << 1) |
-                                   (((V2 >> c) & 1u) << 2) | (((V3 >> c) & 1u) << 3);
-                const unsigned cur = state | 8u;
-                const unsigned nxt = (__popc(v) < __popc(cur)) ? v : cur;
-                ones += (int)(nxt & 1u);
-                state = nxt >> 1;
+            // columns past the end: a vector without ones, whose final bit is 0
+            const uint32_t valid = 0xffffffffu >> (32 - ncol);
+            V0 &= valid; V1 &= valid; V2 &= valid; V3 &= valid;
+            const uint32_t P[4] = {nibbles<0>(V0, V1, V2, V3), nibbles<1>(V0, V1, V2, V3),
+                                   nibbles<2>(V0, V1, V2, V3), nibbles<3>(V0, V1, V2, V3)};
+            unsigned final = 0u;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (k % 2 == 0 && 4 * k >= ncol) break;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const uint32_t t = steps[(P[j] >> (4 * k)) & 15u];
+                    const uint32_t r = __funnelshift_r(t, t, state);
+                    state = r & 28u;
+                    final += r & 32u;
+                }
             }
+            ones += (int)(final >> 5);
             x.next(a.pairs);
 #pragma unroll
             for (int k = 0; k < NSMAX; ++k)
                 if (k < ns) {
                     A[k] = B[k];
-                    B[k] = x.map(k - E);
+                    B[k] = x.row(k);
                 }
         }
         variant_out(a, p, E, ones);
