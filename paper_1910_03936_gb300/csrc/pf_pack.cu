@@ -85,22 +85,25 @@ __device__ __forceinline__ void decode_chunks(uintptr_t cbase, int nchunks, uint
 // that groups sequences by threshold and length); the block lays its
 // sequences' ceil(len/32) words out locally (a prefix sum by one warp) and
 // writes word w of sequence s to word_off[s] + w.
-constexpr int kSeqPerBlock = 256;
-constexpr int kMapCap = 16 * kSeqPerBlock;
+//
+// SEQS sequences a block: 256, or 64 for few sequences, where blocks of 256
+// leave SMs without work and walk their words in five rounds (kFewSeqs).
+constexpr int kSeqPerBlock = 256, kFewSeqPerBlock = 64;
 
 // Six blocks per SM: at eight the kernel's 32 registers spill.
-template <bool STARTS>
+template <bool STARTS, int SEQS>
 __global__ void __launch_bounds__(kPackThreads, 6)
 pack_ragged_kernel(const uint8_t *ascii, const int64_t *byte_off, const int64_t *word_off,
                    int64_t nseq, uint32_t *lo, uint32_t *hi, uint32_t *nm, unsigned *err,
                    const int32_t *seg_of, unsigned *seg_err) {
-    __shared__ int woff[kSeqPerBlock + 1];       // block-local first word, rising
-    __shared__ int64_t wdst[kSeqPerBlock + 1];   // first word in the planes
-    __shared__ int64_t boff[kSeqPerBlock + 1];
-    __shared__ int32_t sseg[kSeqPerBlock];
+    constexpr int kMapCap = 16 * SEQS;
+    __shared__ int woff[SEQS + 1];       // block-local first word, rising
+    __shared__ int64_t wdst[SEQS + 1];   // first word in the planes
+    __shared__ int64_t boff[SEQS + 1];
+    __shared__ int32_t sseg[SEQS];
     __shared__ uint8_t wseq[kMapCap];            // local word -> local sequence
-    const int64_t s0 = (int64_t)blockIdx.x * kSeqPerBlock;
-    const int ns = (int)min((int64_t)kSeqPerBlock, nseq - s0);
+    const int64_t s0 = (int64_t)blockIdx.x * SEQS;
+    const int ns = (int)min((int64_t)SEQS, nseq - s0);
     for (int i = threadIdx.x; i <= ns; i += blockDim.x) {
         boff[i] = byte_off[s0 + i];
         if (!STARTS || i < ns) wdst[i] = word_off[s0 + i];
@@ -108,7 +111,7 @@ pack_ragged_kernel(const uint8_t *ascii, const int64_t *byte_off, const int64_t 
     }
     __syncthreads();
     if constexpr (STARTS) {
-        constexpr int PER = kSeqPerBlock / 32;
+        constexpr int PER = SEQS / 32;
         if (threadIdx.x < 32) {
             const int lane = threadIdx.x;
             int c[PER];
@@ -132,7 +135,7 @@ pack_ragged_kernel(const uint8_t *ascii, const int64_t *byte_off, const int64_t 
                 woff[lane * PER + k] = run;
                 run += c[k];
             }
-            if (lane == 31) woff[kSeqPerBlock] = inc;
+            if (lane == 31) woff[SEQS] = inc;
         }
     } else {
         for (int i = threadIdx.x; i <= ns; i += blockDim.x) woff[i] = (int)(wdst[i] - wdst[0]);
@@ -281,6 +284,23 @@ pack_stream_kernel(const uint8_t *ascii, int64_t nseq, int len, int W, uint32_t 
     }
 }
 
+// Below, 64 sequences a block.  Pack, filter and verification of 1000 mixed
+// pairs: 64.7 us with 256, 57.3 with 64; 16,000: 87.9 and 83.9; 50,000: 131.8
+// and 130.7; 100,000: 150.8 and 151.5; 500,000: 327 and 342.
+constexpr int64_t kFewSeqs = 50000;
+
+template <bool STARTS>
+void launch_ragged(const uint8_t *ascii, const int64_t *byte_off, const int64_t *word_off,
+                   int64_t nseq, uint32_t *lo, uint32_t *hi, uint32_t *nm, unsigned *err,
+                   cudaStream_t st, const int32_t *seg_of, unsigned *seg_err) {
+    const bool few = nseq < kFewSeqs;
+    const int per = few ? kFewSeqPerBlock : kSeqPerBlock;
+    const auto kernel = few ? pack_ragged_kernel<STARTS, kFewSeqPerBlock>
+                            : pack_ragged_kernel<STARTS, kSeqPerBlock>;
+    kernel<<<(unsigned)((nseq + per - 1) / per), kPackThreads, 0, st>>>(
+        ascii, byte_off, word_off, nseq, lo, hi, nm, err, seg_of, seg_err);
+}
+
 }  // namespace
 
 cudaError_t launch_pack_ragged(const uint8_t *ascii, const int64_t *byte_off,
@@ -288,9 +308,7 @@ cudaError_t launch_pack_ragged(const uint8_t *ascii, const int64_t *byte_off,
                                uint32_t *hi, uint32_t *nm, unsigned *err, cudaStream_t st,
                                const int32_t *seg_of, unsigned *seg_err) {
     if (nseq <= 0) return cudaSuccess;
-    const int64_t blocks = (nseq + kSeqPerBlock - 1) / kSeqPerBlock;
-    pack_ragged_kernel<false><<<(unsigned)blocks, kPackThreads, 0, st>>>(
-        ascii, byte_off, word_off, nseq, lo, hi, nm, err, seg_of, seg_err);
+    launch_ragged<false>(ascii, byte_off, word_off, nseq, lo, hi, nm, err, st, seg_of, seg_err);
     return cudaGetLastError();
 }
 
@@ -298,9 +316,7 @@ cudaError_t launch_pack_starts(const uint8_t *ascii, const int64_t *byte_off,
                                const int64_t *word_start, int64_t nseq, uint32_t *lo,
                                uint32_t *hi, uint32_t *nm, unsigned *err, cudaStream_t st) {
     if (nseq <= 0) return cudaSuccess;
-    const int64_t blocks = (nseq + kSeqPerBlock - 1) / kSeqPerBlock;
-    pack_ragged_kernel<true><<<(unsigned)blocks, kPackThreads, 0, st>>>(
-        ascii, byte_off, word_start, nseq, lo, hi, nm, err, nullptr, nullptr);
+    launch_ragged<true>(ascii, byte_off, word_start, nseq, lo, hi, nm, err, st, nullptr, nullptr);
     return cudaGetLastError();
 }
 
