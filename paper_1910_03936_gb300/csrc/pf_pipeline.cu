@@ -1,4 +1,4 @@
-// a7: the whole path on host buffers, in chunks, replayed as CUDA graphs.
+// a7: the whole path on host buffers, in chunks.
 // Contract: pf_run_host in pf.h.
 //
 // Two slots alternate.  A slot has device buffers for one chunk (ASCII,
@@ -212,8 +212,6 @@ pf_status enqueue_chunk(Job &J, Slot &s, int64_t nc) {
 }
 
 pf_status capture(Job &J, Slot &s, int64_t nc, cudaGraphExec_t *exec) {
-    // occupancy queries before the capture
-    for (int c = 0; c < kNumBatchCfgs; ++c) J.ctx->grid_for((int)J.dec, c);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(s.st, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return J.ctx->cuda(e, "pf_run_host capture");
@@ -286,7 +284,17 @@ extern "C" pf_status pf_run_host(pf_ctx *ctx, unsigned deciders, const uint8_t *
     }
     Slot slots[2];
     pf_status st = PF_OK;
+    // occupancy queries (the first of a kernel loads it) and captures before the
+    // first upload
+    for (int e = E ? 0 : E_max; e <= E_max; ++e) {
+        const int c = ctx->tune_cfg[deciders][e];
+        if (c >= 0) ctx->grid_for((int)deciders, c);
+    }
     const bool replay = n / J.C >= kGraphChunks;
+    for (int i = 0; i < 2 && replay && st == PF_OK; ++i) {
+        st = setup_slot(J, slots[i], i);
+        if (st == PF_OK) st = capture(J, slots[i], J.C, &slots[i].exec);
+    }
     for (int64_t c = 0; c < nchunks && st == PF_OK; ++c) {
         Slot &s = slots[c & 1];
         if (!s.st) {
@@ -309,9 +317,7 @@ extern "C" pf_status pf_run_host(pf_ctx *ctx, unsigned deciders, const uint8_t *
                             s.st);
         if (E) cudaMemcpyAsync(s.E, E + c0, (size_t)nc * 2, cudaMemcpyHostToDevice, s.st);
         if (replay && nc == J.C) {
-            if (!s.exec) st = capture(J, s, nc, &s.exec);
-            if (st == PF_OK)
-                st = ctx->cuda(cudaGraphLaunch(s.exec, s.st), "pf_run_host graph launch");
+            st = ctx->cuda(cudaGraphLaunch(s.exec, s.st), "pf_run_host graph launch");
         } else {
             st = enqueue_chunk(J, s, nc);
         }
