@@ -431,9 +431,9 @@ PF_API pf_status pf_host_free(void *ptr);
 
 /* Pack, filter, compact and verify n pairs held in HOST memory, chunk by
  * chunk: two slots with their own device buffers and streams alternate,
- * so one chunk's upload overlaps the other's device work; each slot's
- * device work (offsets, pack, filter, compaction, verification) is captured
- * once as a CUDA graph and replayed for every chunk of that size.  Returns
+ * so one chunk's upload overlaps the other's device work (offsets, pack,
+ * filter, compaction, verification); from eight full chunks on each slot's is
+ * captured once as a CUDA graph and replayed for every full chunk.  Returns
  * when every result is in host memory.
  *   reads, refs  host ASCII; pair p is bytes [byte_off[p], byte_off[p+1])
  *                of both (host int64[n+1]) or, when byte_off is NULL,
@@ -443,7 +443,8 @@ PF_API pf_status pf_host_free(void *ptr);
  *   chunk_pairs  pairs per chunk (>= 1; 0 = 2^20)
  * Page-locked host buffers (pf_host_alloc's, or any registered memory)
  * are copied asynchronously; pageable ones work but serialise the copies.
- * Allocates its slot buffers (freed on return). */
+ * Allocates its slot buffers; they stay with the context for later calls up to
+ * 1 GiB a slot (larger ones are freed on return) and are freed by pf_destroy. */
 PF_API pf_status pf_run_host(pf_ctx *ctx, unsigned deciders, const uint8_t *reads,
                              const uint8_t *refs, const int64_t *byte_off, int len,
                              const int16_t *E, int E_max, uint8_t *accept, int16_t *count,

@@ -1,4 +1,4 @@
-// a6: verification kernel, one thread per pair (device function and its
+// a6: verification kernel, one or two pairs per thread (device functions and their
 // derivation in pf_verify.cuh).
 #include <algorithm>
 
@@ -80,7 +80,7 @@ __device__ __forceinline__ void verify_chunk(const PairsView &pv, const int32_t 
 // each has by its number, from the last position on: when the indices come
 // grouped by threshold and length, the costly groups lie together at the end,
 // and a fixed assignment would leave them to a few blocks.  The claims of one
-// address take 2.9 ns each, so the grid is what is resident and the next claim
+// address take 2.9 ns each, so the grid is about what is resident and the next claim
 // is under way while a chunk is verified: with a claim for every chunk by 1216
 // blocks, 0.63M pairs of 150 bp, E = 6, took 80 us more.
 template <Bands B>
@@ -119,9 +119,10 @@ cudaError_t launch_verify(const PairsView &pv, const int32_t *lens, const int16_
     if (n <= 0) return cudaSuccess;
     const bool two = E_max <= kTwoE && n >= kTwoFrom;
     if (!E) work = nullptr;  // one threshold: no group is costlier
-    // 24 warps an SM are resident; striding ones come in several waves, which
-    // levels their ends (2M pairs, E = 6: 64 warps an SM 5 % faster than 24).
-    // Few pairs spread over the SMs in blocks of two warps.
+    // 16 to 24 warps an SM are resident (16, 20 and 24 take the same for claims);
+    // striding ones come in several waves, which levels their ends (2M pairs,
+    // E = 6: 64 warps an SM 5 % faster than 24).  Few pairs spread over the SMs
+    // in blocks of two warps.
     const int threads = n < kTwoFrom ? 64 : 256;
     const int64_t cap = (int64_t)sms * (work ? 24 : 64) * 32 / threads;
     const int64_t per = two ? 2 * threads : threads;

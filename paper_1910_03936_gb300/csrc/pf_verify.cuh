@@ -4,7 +4,8 @@
 // Levenshtein distance (Ch. 2, "Accelerating Read Alignment": Ukkonen's
 // band of 2E+1 diagonals).  This kernel computes that band with bit
 // vectors: one machine word holds the vertical differences of the 2E+1
-// band cells of a DP column (Myers 1999; Hyyrö 2003), one thread per pair.
+// band cells of a DP column (Myers 1999; Hyyrö 2003), one thread per pair (or
+// two pairs, further down).
 //
 // Rows are read prefixes (row i = read[0..i)), columns reference prefixes.
 // Column j keeps the cells of rows j-E .. j+E as
