@@ -67,11 +67,12 @@ __device__ __forceinline__ void verify_chunk(const PairsView &pv, const int32_t 
             return;
         }
     }
-    if (B == Bands::kTwo) return;
+    if constexpr (B != Bands::kTwo) {
 #pragma unroll 1
-    for (int k = 0; k < (two ? 2 : 1); ++k) {
-        verify_one<B>(pv, a, dist);
-        a = b;
+        for (int k = 0; k < (two ? 2 : 1); ++k) {
+            verify_one<B>(pv, a, dist);
+            a = b;
+        }
     }
 }
 
