@@ -247,8 +247,8 @@ struct SliceColumns {
     bool even;                  // the tile's pairs lie one stride apart
     int64_t rbase, fbase;       // even: first word of the tile's first pair,
     uint32_t rstep, fstep;      // words from a pair to the next
-    int64_t *rstart, *fstart;   // else first words of the pairs, in shared memory
-                                // (launches over a strided layout in pair order have none)
+    int64_t *rstart, *fstart;   // else first words of the pairs, in shared memory (launches
+                                // over two strided sides in pair order have none)
     int W;              // words of the tile's longest pair
     int w0, nr, nf;     // the next segment's words: first of each side, counts
     int r0;
@@ -261,12 +261,20 @@ struct SliceColumns {
         rn = reinterpret_cast<uint32_t *>(fx + FC * G);
         fn = rn + RC * G;
         W = (sp.mmax + 31) >> 5;
-        // starts are looked up once: a pair's words are loaded in many rounds
-        const int lane = threadIdx.x & 31;
+        even = true;
+        if (!order && slice_strided(pv.read) && slice_strided(pv.ref)) {
+            rbase = pos * pv.read.stride;
+            fbase = pos * pv.ref.stride;
+            rstep = (uint32_t)pv.read.stride;
+            fstep = (uint32_t)pv.ref.stride;
+            return;
+        }
+        // starts are looked up once: a pair's words are loaded in many rounds.
+        // Both sides have tables here, a strided one too: where one side is not
+        // even, both are loaded by them.
         const bool same = slice_same(pv);
         rstart = reinterpret_cast<int64_t *>(sm + slice_smem_words(L));
         fstart = rstart + (same ? 0 : 32 * G);
-        even = true;
         place(pv.read, sp, order, pos, rstart, rbase, rstep);
         if (same) {
             fbase = rbase;
@@ -277,16 +285,11 @@ struct SliceColumns {
         even = __all_sync(0xffffffffu, even);
     }
 
-    // Where one side's pairs lie: evenly spaced (the strided layout, and a
-    // ragged one whose neighbours here are neighbours in memory), or a table.
+    // Where one side's pairs lie: a table, and whether they are evenly spaced
+    // (neighbours here are neighbours in memory).
     __device__ __forceinline__ void place(const SeqView &v, const SlicePairs<L> &sp,
                                           const int64_t *order, int64_t pos, int64_t *table,
                                           int64_t &base, uint32_t &step) {
-        if (!order && !v.off && v.stride < (1 << 24)) {
-            base = pos * v.stride;
-            step = (uint32_t)v.stride;
-            return;
-        }
         const int lane = threadIdx.x & 31;
         int64_t st[G];
 #pragma unroll
