@@ -82,9 +82,10 @@ __host__ __device__ constexpr size_t slice_smem_words(int L) {
     return (size_t)3 * (32 / L) *
            (32 * (slice_seg(L) + 2) + slice_block(L) - 1 + 32 * slice_seg(L));
 }
-// A side whose words are found by a 32-bit step from pair to pair.
+// A side whose words are found by an unsigned 32-bit step from pair to pair (rows
+// may also run backwards: pf_filter_partitioned takes negative strides).
 __host__ __device__ constexpr bool slice_strided(const SeqView &v) {
-    return !v.off && v.stride < (1 << 24);
+    return !v.off && v.stride >= 0 && v.stride < (1 << 24);
 }
 // and the bytes with the starts of its pairs where the launch needs them (the
 // smaller, the more L1 is left for the loads: 0.36 against 0.39 ms for 4M pairs

@@ -117,3 +117,32 @@ def test_submatrices(pf, sides, n):  # noqa: F811
             assert np.array_equal(acc.cpu().numpy(), (want <= E).astype(np.uint8))
     finally:
         pf.pf_destroy(c)
+
+
+@pytest.mark.parametrize("n", [300, 200003])
+@pytest.mark.parametrize("both", [False, True])
+def test_submatrices_over_rows_that_run_backwards(pf, n, both):  # noqa: F811
+    """pf_filter_partitioned takes a negative stride; the rows lie in reverse
+    behind the planes' first one."""
+    c = pf.pf_create(0)
+    try:
+        E = 9
+        P, pairs, rep = batch(pf, c, 77, n, E)
+        want = oracle.int_batch("ss_partitioned", P, p0=8, p1=2)[rep]
+
+        def backwards(seqs):
+            fwd = moved(pf, seqs, n, "strided")
+            planes = [x.view(n, W).flip(0).reshape(-1) for x in (fwd.lo, fwd.hi, fwd.nmask)]
+            return pf.Seqs(*[x[(n - 1) * W:] for x in planes], stride_words=-W)
+
+        read = backwards(pairs.read)
+        ref = backwards(pairs.ref) if both else moved(pf, pairs.ref, n, "strided")
+        lens = torch.full((n,), M, dtype=torch.int32, device=DEV)
+        acc = torch.full((n,), 9, dtype=torch.uint8, device=DEV)
+        cnt = torch.full((n,), 99, dtype=torch.int16, device=DEV)
+        pf.pf_filter_partitioned(c, pf.Pairs(read, ref), lens, None, E, 8, 2, acc, cnt, n)
+        pf.pf_sync(c)
+        assert np.array_equal(cnt.cpu().numpy(), want)
+        assert np.array_equal(acc.cpu().numpy(), (want <= E).astype(np.uint8))
+    finally:
+        pf.pf_destroy(c)
