@@ -34,6 +34,11 @@
 // per 1,024-pair tile (0.29 ms for SneakySnake, 0.42 against 0.36 ms with
 // both deciders).
 //
+// A tile ends with the segment after which all of its pairs are decided.  The vote
+// costs up to 1 % where pairs are short and some accepted (250 bp, E = 25, whole
+// path: 0.697 -> 0.702 ms); 2M unrelated pairs of 300 bp at E = 8, both deciders:
+// 0.46 -> 0.16 ms, 0.3M of 5,000 bp 2.0 -> 0.1.
+//
 // Both deciders, ms, word-per-pair kernels -> this one: 4M pairs of 150 bp at
 // E = 6 0.44 -> 0.35, E = 8 0.58 -> 0.39, E = 15 1.50 -> 0.50; 2M pairs of 250 bp
 // at E = 8 0.48 -> 0.34, E = 20 1.75 -> 0.52, E = 25 2.12 -> 0.56.
@@ -133,6 +138,17 @@ struct VCount {
 #pragma unroll
         for (int i = 0; i < NB; ++i) b[i] = __shfl_sync(0xffffffffu, b[i], src);
     }
+    // the pairs whose count is past E
+    __device__ __forceinline__ uint32_t above(int E) const {
+        uint32_t gt = sat, eq = 0xffffffffu;
+#pragma unroll
+        for (int i = NB - 1; i >= 0; --i) {
+            const uint32_t e = 0u - (uint32_t)((E >> i) & 1);
+            gt |= eq & b[i] & ~e;
+            eq &= ~(b[i] ^ e);
+        }
+        return gt;
+    }
     // pair l's count, at most top
     __device__ __forceinline__ int get(int l, int top) const {
         int v = 0;
@@ -177,7 +193,8 @@ struct SlicePairs {
     int m[G];           // length; -1: absent or invalid
     unsigned invalid;   // bit t: present but its arguments are bad
     int mmin, mmax;     // over the tile's valid pairs (0 when there are none)
-    bool whole;         // all 32 * G pairs present and valid, of one length in words
+    bool full;          // all 32 * G pairs present and valid
+    bool whole;         // and of one length in words
 
     __device__ __forceinline__ int64_t pair(const int64_t *order, int64_t pos, int t) const {
         const int64_t s = pos + 32 * t + (threadIdx.x & 31);
@@ -189,7 +206,7 @@ struct SlicePairs {
         const int lane = threadIdx.x & 31;
         invalid = 0u;
         int lo = INT_MAX, hi = 0, wlo = INT_MAX, whi = 0;
-        bool all = cnt == 32 * G;
+        full = cnt == 32 * G;
 #pragma unroll
         for (int t = 0; t < G; ++t) {
             m[t] = -1;
@@ -199,7 +216,7 @@ struct SlicePairs {
                 const int e = Es ? (int)__ldg(Es + p) : E_max;
                 if (len < 0 || e != E || e > E_max) {
                     invalid |= 1u << t;
-                    all = false;
+                    full = false;
                 } else {
                     m[t] = len;
                     lo = min(lo, len);
@@ -211,9 +228,9 @@ struct SlicePairs {
         mmax = __reduce_max_sync(0xffffffffu, hi);
         wlo = (mmin + 31) >> 5;
         whi = (mmax + 31) >> 5;
-        all = __all_sync(0xffffffffu, all);
+        full = __all_sync(0xffffffffu, full);
         if (mmin > mmax) mmin = mmax;  // no valid pair
-        whole = all && wlo == whi;
+        whole = full && wlo == whi;
     }
 
     // bit of every pair of the group that has a column i
@@ -588,6 +605,25 @@ struct SliceWalk {
             xn[j] = xn[j + U];
         }
     }
+
+    // Whether columns from i on can change nothing: every pair that has them
+    // (GateKeeper's counts lag `extra` columns) is past E by each decider.
+    __device__ __forceinline__ bool decided(const SlicePairs<L> &sp, int E, int i, int extra) const {
+        uint32_t open = 0xffffffffu;
+        if (!sp.full || i - extra >= sp.mmin) open = sp.valid(i - extra);
+        if constexpr (SS)
+            if (__any_sync(0xffffffffu, open & ~ss.above(E))) return false;
+        if constexpr (GK) {
+            const int g = (threadIdx.x & 31) % G;
+            const uint32_t h = __shfl_sync(0xffffffffu, hm.above(E), S::H * G + g);
+            if (__any_sync(0xffffffffu, open & ~h)) return false;
+            VCount<S::NB> sum = gk;
+#pragma unroll
+            for (int x = G; x < 32; x <<= 1) sum.add_lane(x);
+            if (__any_sync(0xffffffffu, open & ~sum.above(E))) return false;
+        }
+        return true;
+    }
 };
 
 // Walk a tile's columns: positions [pos, pos + cnt) of a bin whose pairs all
@@ -624,6 +660,10 @@ __device__ __forceinline__ void slice_walk(const FilterArgs &a, const SlicePairs
             }
             w.block(c, f, v);
         }
+        // (an obstacle of unrelated pairs comes every four columns or more; the
+        // last words are not worth a vote)
+        const int i = i0 + 32 * SEG;
+        if (i >= 3 * E && total - i >= 64 && w.decided(sp, E, i, extra)) break;
     }
 }
 
