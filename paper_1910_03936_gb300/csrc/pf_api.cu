@@ -23,7 +23,9 @@ struct BinTable {
 };
 
 __global__ void bin_init_kernel(int64_t *bin_start, unsigned long long *work,
-                                unsigned long long *hist, int nb, int single_cfg, int64_t n) {
+                                unsigned long long *hist, int64_t *late, int nb, int single_cfg,
+                                int64_t n) {
+    if (threadIdx.x < 3) late[threadIdx.x] = 0;
     for (int i = threadIdx.x; i <= nb; i += blockDim.x) {
         bin_start[i] = (single_cfg >= 0) ? (i <= single_cfg ? 0 : n) : 0;
         if (i < nb) work[i] = 0ull;
@@ -191,7 +193,8 @@ bin_scatter_kernel(const int16_t *E, const int32_t *lens, int64_t n, int E_max, 
 // Group the pairs: bin t.cfg_of_E[E], E clamped to [0, E_max], of nbins bins.
 static cudaError_t launch_binning(const FilterArgs &a, const BinTable &t, int nbins,
                                   const Scratch &s, int sms, cudaStream_t st) {
-    bin_init_kernel<<<1, 256, 0, st>>>(s.bin_start, s.work, s.hist, kNumBatchCfgs, -1, a.n);
+    bin_init_kernel<<<1, 256, 0, st>>>(s.bin_start, s.work, s.hist, s.late(), kNumBatchCfgs, -1,
+                                       a.n);
     const int64_t hh = std::max<int64_t>(
         1, std::min<int64_t>((a.n + 256 * kHistPer - 1) / (256 * kHistPer), (int64_t)sms * 8));
     bin_hist_kernel<<<(unsigned)hh, 256, 0, st>>>(a.E, a.lens, a.n, a.E_max, t, s.hist);
@@ -277,7 +280,7 @@ pf_status pf_ctx::scratch_layout(int64_t n, Scratch *s) {
     const size_t o_work = off;  off += up(kWorkCounters * sizeof(unsigned long long));
     const size_t o_hist = off;  off += up(kNumBinKeys * sizeof(unsigned long long));
     const size_t o_cur = off;   off += up(kNumBinKeys * sizeof(unsigned long long));
-    const size_t o_ident = off; off += up(2 * sizeof(int));
+    const size_t o_ident = off; off += up(kFlagBytes);
     const size_t o_need = off;  off += up(nn);
     pf_status st = ensure_scratch(off);
     if (st != PF_OK) return st;
@@ -308,7 +311,7 @@ int pf_ctx::grid_for(int dec, int cfg) {
 }
 
 // Default configuration for threshold E before any tuning.  The bit-sliced
-// kernels from the threshold on at which they win whatever the lengths (in a
+// kernels from the threshold on at which they win for pairs up to long_words (in a
 // tile of mixed lengths every pair is walked to the longest one's end; the
 // tuner finds them lower down where lengths agree).  Filter, ms, best
 // word-per-pair kernel -> bit-sliced: 3M pairs of 100/150/250 bp mixed in pair order,
@@ -327,6 +330,35 @@ int pf::pf_default_cfg(int dec, int E) {
         for (int c = 0; c < kNumBatchCfgs; ++c)
             if (kBatchCfgs[c].xe == E && kBatchCfgs[c].words >= 8) return c;
     return kFirstExactCfg + E;
+}
+
+// The word-per-pair configuration for the long pairs of threshold E: the exact
+// one, or from E = 16 on two or four lanes with the fewest slots that hold the
+// 2E + 1 diagonals (four on a tie); each: pairs of thresholds up to E.
+int pf::pf_long_cfg(int E, bool each) {
+    if (each) return E <= 15 ? kTwoLaneCfg : kFourLaneCfg;
+    if (E <= 15) return kFirstExactCfg + E;
+    int best = -1;
+    for (int c = 0; c < kNumBatchCfgs; ++c) {
+        const KernelCfg &k = kBatchCfgs[c];
+        if ((k.tpp != 2 && k.tpp != 4) || k.xe >= 0 || k.ecap < E || k.words < 8) continue;
+        if (best < 0 || k.ecap < kBatchCfgs[best].ecap ||
+            (k.ecap == kBatchCfgs[best].ecap && k.tpp > kBatchCfgs[best].tpp))
+            best = c;
+    }
+    return best;
+}
+
+// Whether bit-sliced launches for thresholds from E on may meet long pairs.
+static bool may_be_long(const FilterArgs &a, int E) { return row_words(a.pairs) >= long_words(E); }
+
+// All pairs are probably long: strided rows of as many words.
+static bool long_rows(const FilterArgs &a, int E) {
+    return may_be_long(a, E) && row_words(a.pairs) < INT64_MAX;
+}
+
+static LongPairs list_of(const Scratch &s) {
+    return {true, s.idx, reinterpret_cast<unsigned long long *>(s.late() + 1)};
 }
 
 // E = 0 compares one diagonal and is bound by memory: the plain kernel
@@ -401,6 +433,9 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
     int single = -1;
     if (cfg >= 0 || !a.E) {
         single = cfg >= 0 ? cfg : tune_cfg[dec][a.E_max];
+        // rows of long pairs: no tiles that would only list them
+        if (cfg_sliced(kBatchCfgs[single]) && kBatchCfgs[single].tpp == 4 && long_rows(a, a.E_max))
+            single = pf_long_cfg(a.E_max, false);
         used.push_back(single);
         b.order = nullptr;
     } else {
@@ -422,8 +457,8 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
         for (int e = 0; e <= PF_MAX_E; ++e) t.cfg_of_E[e] = tune_cfg[dec][std::min(e, a.E_max)];
         st = cuda(launch_binning(a, t, kNumBatchCfgs, s, sms, stream), "binning launch");
     } else {
-        bin_init_kernel<<<1, 256, 0, stream>>>(s.bin_start, s.work, s.hist, kNumBatchCfgs, single,
-                                               a.n);
+        bin_init_kernel<<<1, 256, 0, stream>>>(s.bin_start, s.work, s.hist, s.late(),
+                                               kNumBatchCfgs, single, a.n);
         st = cuda(cudaGetLastError(), "binning launch");
     }
     if (st != PF_OK) return st;
@@ -439,25 +474,38 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
         const int wpb = cfg_threads(kBatchCfgs[c], (int)dec) / 32;  // warps per block
         const int grid = (int)std::min<int64_t>(grid_for(dec, c),
                                                 std::max<int64_t>(1, (steps + wpb - 1) / wpb));
-        return cuda(launch_filter_batched(dec, c, grid, b, c, stream), "filter launch");
+        const bool list = cfg_sliced(kBatchCfgs[c]) && kBatchCfgs[c].tpp == 4 &&
+                          may_be_long(a, kBatchCfgs[c].xe);
+        if (list) b.late = list_of(s);
+        st = cuda(launch_filter_batched(dec, c, grid, b, c, stream), "filter launch");
+        return st == PF_OK && list ? run_late(dec, a, s) : st;
     }
     // Several configurations: one persistent launch each, concurrently.  Where
     // that leaves the average bin less than a wave of bit-sliced tiles (12
     // warps of 256 pairs per SM), the bit-sliced ones share a launch per class.
     // Pairs scattered over the planes (and batches too short for whole classes)
     // take the launch with 16 lanes per group instead, whose segments hold four
-    // words of a pair.  Filter with both deciders, ms, launch per threshold /
-    // per class / 16 lanes: thresholds 0..25, grouped layout, 1.1M pairs 0.65 /
-    // 0.43 / 0.37, 3M 0.94 / 0.71 / 0.91; in pair order 3M 2.57 / 2.22 / 1.02; 1.1M
-    // pairs of eight thresholds up to 20, grouped 0.35 / 0.30 / 0.31.
-    SliceBins sliced{};
+    // words of a pair, and up to E = 10 the word-per-pair kernels.  Filter with
+    // both deciders, ms, launch per threshold / per class / 16 lanes: thresholds
+    // 0..25, grouped layout, 1.1M pairs 0.65 / 0.43 / 0.37, 3M 0.94 / 0.71 / 0.91; in
+    // pair order 3M 2.57 / 2.22 / 1.02; 1.1M pairs of eight thresholds up to 20,
+    // grouped 0.35 / 0.30 / 0.31.  16 lanes / word kernels, pair order: 1.5M pairs
+    // all of E = 8 0.47 / 0.33; 3M of 0..7 0.89 / 0.83.
+    constexpr int kWordsTo = 10;
+    SliceBins sliced{}, wide{};
+    auto add = [](SliceBins &to, int c, int e) {
+        to.bin[to.count] = (unsigned char)c;
+        to.E[to.count++] = (unsigned char)e;
+    };
     for (int e = 0; e <= a.E_max; ++e) {
         const int c = tune_cfg[dec][e];
         if (!cfg_sliced(kBatchCfgs[c])) continue;
-        sliced.bin[sliced.count] = (unsigned char)c;
-        sliced.E[sliced.count++] = (unsigned char)e;
+        add(sliced, c, e);
+        if (e > kWordsTo) add(wide, c, e);
     }
     const bool few = a.n < 1600000;
+    const bool list = (few ? wide.count : sliced.count) && may_be_long(a, sliced.E[0]);
+    if (list) b.late = list_of(s);
     if (sliced.count && !few) {
         bin_layout_kernel<<<1, 1024, 0, stream>>>(a.pairs.read, a.lens, s.order, s.ident, a.n,
                                                   s.ident + 1);
@@ -471,26 +519,29 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
         if (next++ < kSideStreams) cudaStreamWaitEvent(x, ev_fork, 0);
         return x;
     };
-    if (sliced.count) {
-        b.want = 1;
-        st = cuda(launch_filter_slices((int)dec, 16, b, sliced, -1, sms, side()), "filter launch");
-        b.want = 0;
+    b.want = 1;
+    if (wide.count) {
+        st = cuda(launch_filter_slices((int)dec, 16, b, wide, -1, sms, side()), "filter launch");
         if (st != PF_OK) return st;
     }
-    if (few || merge) {
+    b.want = 0;
+    if (few)
+        used.erase(std::remove_if(used.begin(), used.end(),
+                                  [](int c) { return cfg_sliced(kBatchCfgs[c]); }),
+                   used.end());
+    if (!few && merge) {
         // the larger thresholds first
         for (int cls = kSliceClasses - 1; cls >= 0; --cls) {
             SliceBins bins{};
             for (int i = 0; i < sliced.count; ++i) {
                 const int e = sliced.E[i];
-                if (!few && (e > kSliceClassE[cls] || (cls && e <= kSliceClassE[cls - 1]))) continue;
+                if (e > kSliceClassE[cls] || (cls && e <= kSliceClassE[cls - 1])) continue;
                 const auto at = std::find(used.begin(), used.end(), (int)sliced.bin[i]);
                 if (at == used.end()) continue;
                 used.erase(at);
-                bins.bin[bins.count] = sliced.bin[i];
-                bins.E[bins.count++] = (unsigned char)e;
+                add(bins, sliced.bin[i], e);
             }
-            if (few || !bins.count) continue;
+            if (!bins.count) continue;
             st = cuda(launch_filter_slice_bins((int)dec, cls, b, bins, sms, side()),
                       "filter launch");
             if (st != PF_OK) return st;
@@ -499,17 +550,45 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
     for (const int c : used) {
         BatchArgs bi = b;
         bi.chunk = 256;
+        if (!cfg_sliced(kBatchCfgs[c])) bi.layout = nullptr;
         for (int e = 0; e <= a.E_max; ++e)
             if (tune_cfg[dec][e] == c) bi.chunk = tune_chunk[dec][e];
         const int grid = grid_for(dec, c);
         st = cuda(launch_filter_batched(dec, c, grid, bi, c, side()), "filter launch");
         if (st != PF_OK) return st;
     }
+    b.want = 1;
+    for (int i = 0; i < sliced.count && sliced.E[i] <= kWordsTo; ++i) {
+        BatchArgs bi = b;
+        bi.chunk = 256;
+        const int c = pf_long_cfg(sliced.E[i], false);
+        st = cuda(launch_filter_batched(dec, c, grid_for(dec, c), bi, sliced.bin[i], side()),
+                  "filter launch");
+        if (st != PF_OK) return st;
+    }
     for (int i = 0; i < kSideStreams && i < next; ++i) {
         cudaEventRecord(ev_join[i], side_streams[i]);
         cudaStreamWaitEvent(stream, ev_join[i], 0);
     }
-    return cuda(cudaGetLastError(), "filter launch");
+    st = cuda(cudaGetLastError(), "filter launch");
+    return st == PF_OK && list ? run_late(dec, a, s) : st;
+}
+
+// One persistent launch over the list, whose length is known on the device only.
+pf_status pf_ctx::run_late(unsigned dec, const FilterArgs &a, const Scratch &s) {
+    const int c = pf_long_cfg(a.E_max, a.E != nullptr);
+    BatchArgs b{};
+    b.f = a;
+    b.order = s.idx;
+    b.bin_start = s.late();
+    b.work = reinterpret_cast<unsigned long long *>(s.late() + 2);
+    b.chunk = 256;
+    const int wpb = cfg_threads(kBatchCfgs[c], dec) / 32;
+    const int step = cfg_step(kBatchCfgs[c], dec);
+    const int64_t steps = (a.n + step - 1) / step;
+    const int grid =
+        (int)std::min<int64_t>(grid_for(dec, c), std::max<int64_t>(1, (steps + wpb - 1) / wpb));
+    return cuda(launch_filter_batched(dec, c, grid, b, 0, stream), "filter launch");
 }
 
 // ---------------------------------------------------------------------------
@@ -746,7 +825,11 @@ int pf_ctx::small_route(unsigned dec, const FilterArgs &a) const {
             cfg_sliced(kBatchCfgs[pf_default_cfg((int)dec, a.E_max)]))
             return kSmallBatched;
         if (a.E_max < (gk ? 16 : 8)) return kSmallPlain;
+        if (a.E_max < 16 && long_rows(a, a.E_max)) return kSmallPlain;
         if (a.E_max >= 16 && a.n < 8000) return kSmallWide;
+        // too few tiles for their length: 20,000 pairs of 50,000 bp, E = 20, 4.8 ms with
+        // 16 lanes, 1.8 one by one (30,000 of 4,000 0.40 and 0.39)
+        if (a.n < 40000 && long_rows(a, a.E_max) && row_words(a.pairs) >= 256) return kSmallBatched;
         const int64_t plain_below = a.E_max >= 16   ? 0
                                     : a.E_max >= 12 ? 25000
                                     : a.E_max >= 10 ? 50000
@@ -788,9 +871,18 @@ pf_status pf_ctx::run_filter(unsigned dec, const FilterArgs &a, const Scratch &s
             SliceBins bins{};
             for (int e = 0; e <= a.E_max; ++e) bins.bin[e] = bins.E[e] = (unsigned char)e;
             bins.count = a.E_max + 1;
-            return cuda(launch_filter_slices((int)dec, route, b, bins, a.E ? -1 : a.E_max, sms,
-                                             stream),
-                        "filter launch");
+            // (grouped by threshold and length, long pairs share tiles)
+            const bool list = !a.E && a.E_max < 16 && may_be_long(a, a.E_max);
+            pf_status st = PF_OK;
+            if (list) {
+                b.late = list_of(s);
+                st = cuda(cudaMemsetAsync(s.late(), 0, 3 * sizeof(int64_t), stream), "list");
+            }
+            if (st == PF_OK)
+                st = cuda(launch_filter_slices((int)dec, route, b, bins, a.E ? -1 : a.E_max, sms,
+                                               stream),
+                          "filter launch");
+            return st == PF_OK && list ? run_late(dec, a, s) : st;
         }
     } else {
         plain = true;

@@ -16,15 +16,21 @@ namespace pf {
 struct Scratch {
     int64_t *order, *idx, *n_idx, *tiles, *bin_start;
     unsigned long long *work, *hist, *cursor;
-    int *ident;
+    int *ident;      // ident, the layout flag, then `late` (kFlagBytes)
     uint8_t *need;   // pairs left to verify (see FilterArgs::need)
+    // the list of long pairs, kept in idx: its bounds 0 and count, and the work
+    // counter of the launch over it
+    int64_t *late() const { return reinterpret_cast<int64_t *>(ident + 2); }
 };
+
+constexpr size_t kFlagBytes = 2 * sizeof(int) + 3 * sizeof(int64_t);
 
 struct ServeState;
 
 constexpr int kSideStreams = 4;
 
 int pf_default_cfg(int dec, int E);
+int pf_long_cfg(int E, bool each);
 
 // What pf_run_host keeps between calls for one of its two slots.
 struct HostSlot {
@@ -88,6 +94,8 @@ struct pf_ctx {
     // lanes per group of the bit-sliced small-batch kernel, or one of
     enum { kSmallPlain = 0, kSmallWide = -1, kSmallBatched = -2 };
     int small_route(unsigned dec, const pf::FilterArgs &a) const;
+    // the pairs that bit-sliced launches left in the list of s
+    pf_status run_late(unsigned dec, const pf::FilterArgs &a, const pf::Scratch &s);
     // run_batched, or one launch for a batch below small_batch
     pf_status run_filter(unsigned dec, const pf::FilterArgs &a, const pf::Scratch &s);
 };

@@ -517,6 +517,8 @@ __global__ void __launch_bounds__(256) filter_batched_kernel(BatchArgs b, int bi
         (TPP == 32) ? 0xffffffffu : (((1u << TPP) - 1u) << (lane & ~(TPP - 1)));
     constexpr int GPW = 32 / TPP;  // groups per warp
     const int gid = lane / TPP;
+    if constexpr (XE >= 0)
+        if (b.layout && *b.layout != b.want) return;
     const int64_t lo = b.bin_start[bin], hi = b.bin_start[bin + 1];
     const int64_t chunk = item_pairs(hi - lo, b.chunk, GPW);
     unsigned long long *counter = b.work + bin;

@@ -92,6 +92,23 @@ struct FilterArgs {
     uint8_t *need = nullptr;
 };
 
+// Words from which on a pair of threshold E is long: bit-sliced tiles leave such
+// pairs to the word-per-pair kernels.  Their words lie far apart, and each of
+// the 128-byte lines that a tile of 256 pairs needs for one column of words is
+// gone from L2 before the next column; a few long pairs make a whole tile walk
+// their columns.  1.5M pairs, a fifth accepted, tiles / word kernels, ms:
+// SneakySnake at E = 8 320 bp 0.31 / 0.39, 352 bp 0.44 / 0.45, 480 bp 1.03 / 0.55;
+// both deciders at E = 13 448 bp 0.82 / 1.20, SneakySnake 480 bp 1.02 / 1.00;
+// at E = 20 640 bp 1.84 / 3.08, 1000 bp 3.26 / 1.85 (1M pairs).
+__host__ __device__ constexpr int long_words(int E) { return E < 10 ? 12 : (E < 16 ? 16 : 21); }
+
+// Where a tile leaves its long pairs (off: it walks them).
+struct LongPairs {
+    bool on = false;
+    int64_t *list = nullptr;                // null: another launch finds them by their lengths
+    unsigned long long *count = nullptr;    // zeroed
+};
+
 // Warps per block of the two-phase filter kernel.
 constexpr int kSplitWarps = 4;
 
@@ -108,9 +125,11 @@ struct BatchArgs {
     const int64_t *chunk_start;  // [nbins+1] first work item of each bin
     const int *ident;            // device flag: order is the identity (one bin used)
     // non-null: device flag, 1 when the pairs of a bin are scattered over the
-    // planes; a launch does its work only where the flag equals `want`
+    // planes; a launch (bit-sliced or exact-threshold) does its work only where
+    // the flag equals `want`
     const int *layout = nullptr;
     int want = 0;
+    LongPairs late;              // bit-sliced launches
 };
 
 }  // namespace pf

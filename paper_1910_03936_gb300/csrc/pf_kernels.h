@@ -96,6 +96,13 @@ inline size_t slice_smem_bytes(int L, const BatchArgs &b) {
     const int tables = strided ? 0 : (r.off == f.off && r.stride == f.stride ? 1 : 2);
     return slice_smem_words(L) * sizeof(uint32_t) + tables * 32 * (32 / L) * sizeof(int64_t);
 }
+// Words of the longest pair that the layout allows: strided rows hold no more
+// (rows that overlap or repeat tell nothing).
+inline int64_t row_words(const PairsView &pv) {
+    const SeqView &r = pv.read, &f = pv.ref;
+    const int64_t lo = r.stride < f.stride ? r.stride : f.stride;
+    return r.off || f.off || lo < 1 ? INT64_MAX : (r.stride > f.stride ? r.stride : f.stride);
+}
 // Warps per SM that a kernel's registers are held to.  More warps hide more
 // latency but leave less L1 for the loads (the walk's arrays take 13.6 KB per
 // warp).  SneakySnake, 12 / 9 warps: 0.285 / 0.283 ms for 4M pairs of 150 bp at
@@ -151,6 +158,9 @@ constexpr int kNumBinKeys = kNumBatchCfgs * kLenClasses;
 // then the verifier's.
 constexpr int kWorkCounters = kNumBatchCfgs + 1;
 constexpr int kFirstExactCfg = 20;  // kBatchCfgs[20 + E] serves exactly E
+constexpr int kTwoLaneCfg = 10, kFourLaneCfg = 16;  // E <= 15, every threshold
+static_assert(kBatchCfgs[kTwoLaneCfg].tpp == 2 && kBatchCfgs[kTwoLaneCfg].ecap == 15);
+static_assert(kBatchCfgs[kFourLaneCfg].tpp == 4 && kBatchCfgs[kFourLaneCfg].ecap == PF_MAX_E);
 constexpr int kWideCfg = 19;        // one warp per pair, every threshold
 static_assert(kBatchCfgs[kWideCfg].tpp == 32 && kBatchCfgs[kWideCfg].ecap == PF_MAX_E);
 
@@ -179,8 +189,10 @@ cudaError_t launch_filter_slice_bins(int dec, int cls, const BatchArgs &b, const
 cudaError_t launch_filter_slices(int dec, int lanes, const BatchArgs &b, const SliceBins &bins,
                                  int single, int sms, cudaStream_t st);
 
-// SneakySnake on sub-matrices (t columns, y replications), one threshold.
-cudaError_t launch_submat_sliced(const FilterArgs &a, int t, int y, int sms, cudaStream_t st);
+// SneakySnake on sub-matrices (t columns, y replications), one threshold, 16 or
+// four lanes per group; skip_long: long pairs are left out.
+cudaError_t launch_submat_sliced(const FilterArgs &a, int t, int y, int lanes, bool skip_long,
+                                 int sms, cudaStream_t st);
 
 cudaError_t launch_pack_ragged(const uint8_t *ascii, const int64_t *byte_off,
                                const int64_t *word_off, int64_t nseq, uint32_t *lo,

@@ -111,7 +111,7 @@ pf_status setup_slot(Job &J, Slot &s, int which) {
                  o_tiles = add((size_t)compact_tiles((int64_t)C) * 8),
                  o_bins = add((kNumBatchCfgs + 1) * 8), o_work = add(kWorkCounters * 8),
                  o_hist = add(kNumBinKeys * 8), o_cur = add(kNumBinKeys * 8),
-                 o_ident = add(8), o_need = add(C);
+                 o_ident = add(kFlagBytes), o_need = add(C);
     if (h.bytes < o) {
         release(h);
         if (cudaMalloc(&h.mem, o) != cudaSuccess) {

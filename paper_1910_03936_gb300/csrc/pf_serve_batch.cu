@@ -498,7 +498,7 @@ pf_status batch_start(pf_ctx *ctx, ServeState *Sp) {
                  o_tiles = add((size_t)compact_tiles(P) * 8),
                  o_bins = add((kNumBatchCfgs + 1) * 8), o_work = add(kWorkCounters * 8),
                  o_hist = add(kNumBinKeys * 8), o_cur = add(kNumBinKeys * 8),
-                 o_ident = add(8), o_need = add(nn);
+                 o_ident = add(kFlagBytes), o_need = add(nn);
     size_t o_rd[kBatchSlots], o_rf[kBatchSlots], o_sg[kBatchSlots], o_ro[kBatchSlots],
         o_re[kBatchSlots];
     for (int i = 0; i < kBatchSlots; ++i) {

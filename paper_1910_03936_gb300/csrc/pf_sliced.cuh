@@ -192,6 +192,8 @@ struct SlicePairs {
     static constexpr int G = 32 / L;
     int m[G];           // length; -1: absent or invalid
     unsigned invalid;   // bit t: present but its arguments are bad
+    unsigned late;      // bit t: left out (leave)
+    bool alone;         // for the warp to take one by one
     int mmin, mmax;     // over the tile's valid pairs (0 when there are none)
     bool full;          // all 32 * G pairs present and valid
     bool whole;         // and of one length in words
@@ -201,10 +203,13 @@ struct SlicePairs {
         return order ? __ldg(order + s) : s;
     }
 
+    template <bool FEW>
     __device__ __forceinline__ void load(const int32_t *lens, const int16_t *Es, int E_max, int E,
-                                         const int64_t *order, int64_t pos, int cnt) {
+                                         const int64_t *order, int64_t pos, int cnt,
+                                         const LongPairs &to) {
         const int lane = threadIdx.x & 31;
-        invalid = 0u;
+        invalid = late = 0u;
+        alone = false;
         int lo = INT_MAX, hi = 0, wlo = INT_MAX, whi = 0;
         full = cnt == 32 * G;
 #pragma unroll
@@ -226,11 +231,56 @@ struct SlicePairs {
         }
         mmin = __reduce_min_sync(0xffffffffu, lo);
         mmax = __reduce_max_sync(0xffffffffu, hi);
+        const int most = 32 * (long_words(E) - 1);
+        if (mmax > most) leave<FEW>(order, pos, cnt, E, most, to);
         wlo = (mmin + 31) >> 5;
         whi = (mmax + 31) >> 5;
         full = __all_sync(0xffffffffu, full);
         if (mmin > mmax) mmin = mmax;  // no valid pair
         whole = full && wlo == whi;
+    }
+
+    // The pairs of more than `most` columns leave the tile: into the list, or, in
+    // a tile of FEW (whose batch has no launch to spare), to the tile's own warp one
+    // by one afterwards if they are a few among others.  FEW tiles have more than
+    // four lanes per group and segments long enough for long pairs, which they walk
+    // from E = 16 on faster than the word kernels.
+    template <bool FEW>
+    __device__ __forceinline__ void leave(const int64_t *order, int64_t pos, int cnt, int E,
+                                          int most, const LongPairs &to) {
+        const int lane = threadIdx.x & 31;
+        bool list = to.list != nullptr;
+        if constexpr (FEW) {
+            int n = 0;
+#pragma unroll
+            for (int t = 0; t < G; ++t) n += __popc(__ballot_sync(0xffffffffu, m[t] > most));
+            alone = 8 * n <= cnt;
+            if (!alone && (E >= 16 || !list)) return;
+            if (alone) list = false;
+        } else if (!to.on) {
+            return;
+        }
+        int lo = INT_MAX, hi = 0;
+#pragma unroll
+        for (int t = 0; t < G; ++t) {
+            const uint32_t who = __ballot_sync(0xffffffffu, m[t] > most);
+            if (who && list) {
+                unsigned long long at = 0;
+                if (lane == 0) at = atomicAdd(to.count, (unsigned long long)__popc(who));
+                at = __shfl_sync(0xffffffffu, at, 0);
+                if (m[t] > most) to.list[at + __popc(who & ((1u << lane) - 1u))] = pair(order, pos, t);
+            }
+            if (m[t] > most) {
+                late |= 1u << t;
+                m[t] = -1;
+                full = false;
+            } else if (m[t] >= 0) {
+                lo = min(lo, m[t]);
+                hi = max(hi, m[t]);
+            }
+        }
+        mmin = __reduce_min_sync(0xffffffffu, lo);
+        mmax = __reduce_max_sync(0xffffffffu, hi);
     }
 
     // bit of every pair of the group that has a column i
@@ -667,15 +717,17 @@ __device__ __forceinline__ void slice_walk(const FilterArgs &a, const SlicePairs
     }
 }
 
-template <int L, int DPT, int D>
-__device__ __forceinline__ void filter_sliced_tile(const FilterArgs &a, const int64_t *order,
-                                                   int64_t pos, int cnt, int E, uint32_t *sm) {
+// Returns the bits of the pairs that the warp has to take one by one.
+template <int L, int DPT, int D, bool FEW>
+__device__ __forceinline__ unsigned filter_sliced_tile(const BatchArgs &b, const int64_t *order,
+                                                       int64_t pos, int cnt, int E, uint32_t *sm) {
+    const FilterArgs &a = b.f;
     using S = SliceShape<L, DPT>;
     constexpr int G = S::G;
     const int lane = threadIdx.x & 31;
     const int q = lane / G, g = lane % G;
     SlicePairs<L> sp;
-    sp.load(a.lens, a.E, a.E_max, E, order, pos, cnt);
+    sp.template load<FEW>(a.lens, a.E, a.E_max, E, order, pos, cnt, b.late);
     SliceWalk<L, DPT, D> w;
     // the last amend looks two columns ahead
     slice_walk<L, DPT>(a, sp, order, pos, E, (D & 2) ? 2 : 0, sm, w);
@@ -686,7 +738,7 @@ __device__ __forceinline__ void filter_sliced_tile(const FilterArgs &a, const in
     if constexpr (D & 4) w.hm.from_lane(S::H * G + g);
 #pragma unroll
     for (int t = 0; t < G; ++t) {
-        if (32 * t + lane >= cnt) continue;
+        if (32 * t + lane >= cnt || ((sp.late >> t) & 1u)) continue;
         const int64_t p = sp.pair(order, pos, t);
         if ((sp.invalid >> t) & 1u) {
             write_invalid<D & 3>(a, p);
@@ -700,13 +752,14 @@ __device__ __forceinline__ void filter_sliced_tile(const FilterArgs &a, const in
         if constexpr (D & 2) gkc = h <= E ? h : w.gk.get(l, top);
         write_outputs<D & 3>(a, p, E, ssc, gkc, h);
     }
+    return sp.alone ? sp.late : 0u;
 }
 
 // SneakySnake on sub-matrices of t columns with y replications, the whole batch
 // at threshold a.E_max.
 template <int L, int DPT, int NBY>
 __global__ void __launch_bounds__(32, slice_warps(DPT, false))
-submat_sliced_kernel(FilterArgs a, int t, int y) {
+submat_sliced_kernel(FilterArgs a, int t, int y, LongPairs late) {
     extern __shared__ __align__(16) uint32_t slice_sm[];
     using S = SliceShape<L, DPT>;
     const int lane = threadIdx.x & 31;
@@ -714,7 +767,7 @@ submat_sliced_kernel(FilterArgs a, int t, int y) {
     for (int64_t pos = (int64_t)blockIdx.x * S::TILE; pos < a.n; pos += (int64_t)gridDim.x * S::TILE) {
         const int cnt = (int)min((int64_t)S::TILE, a.n - pos);
         SlicePairs<L> sp;
-        sp.load(a.lens, nullptr, E, E, nullptr, pos, cnt);
+        sp.template load<false>(a.lens, nullptr, E, E, nullptr, pos, cnt, late);
         SliceWalk<L, DPT, 1, NBY> w;
         w.t = t;
         w.y = y;
@@ -722,11 +775,25 @@ submat_sliced_kernel(FilterArgs a, int t, int y) {
         slice_walk<L, DPT>(a, sp, nullptr, pos, E, 0, slice_sm, w);
 #pragma unroll
         for (int k = 0; k < S::G; ++k) {
-            if (32 * k + lane >= cnt) continue;
+            if (32 * k + lane >= cnt || ((sp.late >> k) & 1u)) continue;
             const int64_t p = pos + 32 * k + lane;
             if ((sp.invalid >> k) & 1u) write_invalid<1>(a, p);
             else write_outputs<1>(a, p, E, w.ss.get(k * L + lane / S::G, E + 1), 0, 0);
         }
+    }
+}
+
+// One warp per pair: bit t of a lane's `late` is pair 32 t + lane from pos on.
+template <int DEC>
+__device__ __forceinline__ void slice_alone(const FilterArgs &a, const int64_t *order, int64_t pos,
+                                            unsigned late) {
+    const int lane = threadIdx.x & 31;
+    while (__any_sync(0xffffffffu, late != 0u)) {
+        const int first = late ? 32 * (__ffs(late) - 1) + lane : INT_MAX;
+        const int q = __reduce_min_sync(0xffffffffu, first);
+        const int64_t p = order ? __ldg(order + pos + q) : pos + q;
+        filter_group<32, 2, DEC, -1>(a, p, lane, 0xffffffffu);
+        if (first == q) late &= late - 1u;
     }
 }
 
@@ -746,7 +813,9 @@ filter_sliced_kernel(BatchArgs b, int bin, int E) {
         const int64_t s = lo + (int64_t)item * TILE;
         if (s >= hi) break;
         if (threadIdx.x == 0) next = atomicAdd(b.work + bin, 1ull);  // known when this one is done
-        filter_sliced_tile<L, DPT, D>(b.f, order, s, (int)min((int64_t)TILE, hi - s), E, slice_sm);
+        const int cnt = (int)min((int64_t)TILE, hi - s);
+        const unsigned late = filter_sliced_tile<L, DPT, D, (L > 4)>(b, order, s, cnt, E, slice_sm);
+        if constexpr (L > 4) slice_alone<D & 3>(b.f, order, s, late);
         item = next;
     }
 }
@@ -810,7 +879,7 @@ filter_sliced_bins_kernel(BatchArgs b, SliceBins bins) {
         int cnt;
         // the largest thresholds first: their tiles take longest
         const int E = bins.E[sc.find<TILE>(sc.total - 1 - (int64_t)item, s, cnt)];
-        filter_sliced_tile<4, DPT, D>(b.f, order, s, cnt, E, slice_sm);
+        filter_sliced_tile<4, DPT, D, false>(b, order, s, cnt, E, slice_sm);
         item = next;
     }
 }
@@ -844,15 +913,17 @@ filter_sliced_small_kernel(BatchArgs b, SliceBins bins, int single) {
         const int E = single < 0 ? bins.E[i] : single;
         // diagonals per lane: those of the largest threshold of E's class
         constexpr int H = L / 2;
+        unsigned late = 0u;
         switch (E >> 3) {
             case 0:  // (eight lanes take single thresholds from 8 on only)
                 if constexpr (L > 8)
-                    filter_sliced_tile<L, (7 + H) / H, D>(b.f, order, s, cnt, E, slice_sm);
+                    late = filter_sliced_tile<L, (7 + H) / H, D, true>(b, order, s, cnt, E, slice_sm);
                 break;
-            case 1: filter_sliced_tile<L, (15 + H) / H, D>(b.f, order, s, cnt, E, slice_sm); break;
-            case 2: filter_sliced_tile<L, (23 + H) / H, D>(b.f, order, s, cnt, E, slice_sm); break;
-            default: filter_sliced_tile<L, (31 + H) / H, D>(b.f, order, s, cnt, E, slice_sm); break;
+            case 1: late = filter_sliced_tile<L, (15 + H) / H, D, true>(b, order, s, cnt, E, slice_sm); break;
+            case 2: late = filter_sliced_tile<L, (23 + H) / H, D, true>(b, order, s, cnt, E, slice_sm); break;
+            default: late = filter_sliced_tile<L, (31 + H) / H, D, true>(b, order, s, cnt, E, slice_sm); break;
         }
+        slice_alone<D & 3>(b.f, order, s, late);
     }
 }
 

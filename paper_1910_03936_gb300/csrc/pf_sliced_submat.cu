@@ -8,42 +8,43 @@ namespace pf {
 namespace {
 
 template <int L, int DPT, int NBY>
-cudaError_t go(const FilterArgs &a, int t, int y, int sms, cudaStream_t st) {
+cudaError_t go(const FilterArgs &a, int t, int y, bool skip_long, int sms, cudaStream_t st) {
     BatchArgs b{};
     b.f = a;
     const int64_t tiles = (a.n + SliceShape<L, DPT>::TILE - 1) / SliceShape<L, DPT>::TILE;
     const int64_t grid = std::min<int64_t>(tiles, (int64_t)sms * slice_warps(DPT, false));
-    submat_sliced_kernel<L, DPT, NBY><<<(unsigned)grid, 32, slice_smem_bytes(L, b), st>>>(a, t, y);
+    LongPairs late;
+    late.on = skip_long;
+    submat_sliced_kernel<L, DPT, NBY>
+        <<<(unsigned)grid, 32, slice_smem_bytes(L, b), st>>>(a, t, y, late);
     return cudaGetLastError();
 }
 
 template <int L, int DPT>
-cudaError_t by_y(const FilterArgs &a, int t, int y, int sms, cudaStream_t st) {
-    if (y >= t) return go<L, DPT, 0>(a, t, y, sms, st);
-    if (y <= 3) return go<L, DPT, 2>(a, t, y, sms, st);
-    return go<L, DPT, 5>(a, t, y, sms, st);
+cudaError_t by_y(const FilterArgs &a, int t, int y, bool skip_long, int sms, cudaStream_t st) {
+    if (y >= t) return go<L, DPT, 0>(a, t, y, skip_long, sms, st);
+    if (y <= 3) return go<L, DPT, 2>(a, t, y, skip_long, sms, st);
+    return go<L, DPT, 5>(a, t, y, skip_long, sms, st);
 }
 
 }  // namespace
 
-// Four lanes per group where the tiles fill the GPU (0.47M pairs a wave); 16
-// below, where the length of one tile counts: 250 bp, E = 12, 60,000 pairs take
-// 33 us with 16 lanes, 200,000 take 53 with four.
-cudaError_t launch_submat_sliced(const FilterArgs &a, int t, int y, int sms, cudaStream_t st) {
+cudaError_t launch_submat_sliced(const FilterArgs &a, int t, int y, int lanes, bool skip_long,
+                                 int sms, cudaStream_t st) {
     const int E = a.E_max;
-    if (a.n < 80000) {
-        if (E <= 15) return by_y<16, 2>(a, t, y, sms, st);
-        if (E <= 23) return by_y<16, 3>(a, t, y, sms, st);
-        return by_y<16, 4>(a, t, y, sms, st);
+    if (lanes == 16) {
+        if (E <= 15) return by_y<16, 2>(a, t, y, skip_long, sms, st);
+        if (E <= 23) return by_y<16, 3>(a, t, y, skip_long, sms, st);
+        return by_y<16, 4>(a, t, y, skip_long, sms, st);
     }
-    if (E <= 1) return by_y<4, 1>(a, t, y, sms, st);
-    if (E <= 3) return by_y<4, 2>(a, t, y, sms, st);
-    if (E <= 5) return by_y<4, 3>(a, t, y, sms, st);
-    if (E <= 7) return by_y<4, 4>(a, t, y, sms, st);
-    if (E <= 11) return by_y<4, 6>(a, t, y, sms, st);
-    if (E <= 15) return by_y<4, 8>(a, t, y, sms, st);
-    if (E <= 25) return by_y<4, 13>(a, t, y, sms, st);
-    return by_y<4, 16>(a, t, y, sms, st);
+    if (E <= 1) return by_y<4, 1>(a, t, y, skip_long, sms, st);
+    if (E <= 3) return by_y<4, 2>(a, t, y, skip_long, sms, st);
+    if (E <= 5) return by_y<4, 3>(a, t, y, skip_long, sms, st);
+    if (E <= 7) return by_y<4, 4>(a, t, y, skip_long, sms, st);
+    if (E <= 11) return by_y<4, 6>(a, t, y, skip_long, sms, st);
+    if (E <= 15) return by_y<4, 8>(a, t, y, skip_long, sms, st);
+    if (E <= 25) return by_y<4, 13>(a, t, y, skip_long, sms, st);
+    return by_y<4, 16>(a, t, y, skip_long, sms, st);
 }
 
 }  // namespace pf

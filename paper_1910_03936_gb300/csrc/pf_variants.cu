@@ -24,6 +24,7 @@ struct VariantArgs {
     const int16_t *E;  // null: E_max for every pair
     int E_max;
     int p0, p1;        // t and y, or the SHD flags
+    int shortest = 0;  // partitioned_kernel: pairs of fewer columns are left out
     uint8_t *accept;
     int16_t *count;
     int64_t n;
@@ -108,6 +109,7 @@ __global__ void __launch_bounds__(256) partitioned_kernel(VariantArgs a) {
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < a.n;
          p += (int64_t)gridDim.x * blockDim.x) {
         int m, E;
+        if (a.shortest && __ldg(a.lens + p) < a.shortest) continue;
         if (!variant_args(a, p, &m, &E)) continue;
         const int ns = 2 * E + 1;
         Cursor x;
@@ -544,7 +546,7 @@ extern "C" pf_status pf_filter_partitioned(pf_ctx *ctx, const pf_pairs *pairs,
     if (t < 1 || t > 32 || y < 1) return ctx->fail(PF_EINVAL, "pf_filter_partitioned: t or y");
     if (n == 0) return PF_OK;
     cudaSetDevice(ctx->device);
-    const VariantArgs a = variant_args_of(ctx, pairs, lens, E, E_max, t, y, accept, count, n);
+    VariantArgs a = variant_args_of(ctx, pairs, lens, E, E_max, t, y, accept, count, n);
     // One threshold: bit-sliced tiles, whose time does not depend on t and y.
     // One pair per lane group costs about (E + 2) * steps, steps = 32 y / t per
     // word.  2M pairs of 150 bp, E = 6, t = 8, y = 2 (64): 395 us so, 183 in
@@ -553,9 +555,38 @@ extern "C" pf_status pf_filter_partitioned(pf_ctx *ctx, const pf_pairs *pairs,
     // first take 27 us so and 35 in tiles; 1000 of 250 bp, E = 12, t = 8, y = 2
     // (112) 38 and 28, 30,000 of 150 bp, E = 12, t = 32, y = 4 (56) 19 and 20.
     const int cost = (E_max + 2) * (32 * std::min(y, t) / t);
-    if (!E && (n >= 150000 ? E_max >= 8 || cost >= 18 : E_max >= 8 && cost >= 56))
-        return ctx->cuda(launch_submat_sliced(filter_args_of(a), t, y, ctx->sms, ctx->stream),
-                         "pf_filter_partitioned launch");
+    // Rows of long pairs (long_words): 16 lanes per group or one pair a thread.
+    // 0.33M pairs of 1000 bp, a fifth accepted: E = 8, t = 8, y = 2 545 us in tiles,
+    // 567 one by one; t = 32, y = 1 545 and 295; E = 22 586 and 1431, 586 and 821.
+    // Where lengths are not known, the tiles leave the long pairs to a second launch.
+    const int64_t words = row_words(a.pairs);
+    const bool maybe = words >= long_words(E_max), rows = maybe && words < INT64_MAX;
+    const bool tiles = !E && (n >= 150000 ? E_max >= 8 || cost >= 18 : E_max >= 8 && cost >= 56) &&
+                       !(rows && E_max < 16);
+    if (tiles) {
+        // Four lanes per group where the tiles fill the GPU (0.47M pairs a wave);
+        // 16 below, where the length of one tile counts: 250 bp, E = 12, 60,000
+        // pairs take 33 us with 16 lanes, 200,000 take 53 with four.
+        const int lanes = n < 80000 || rows ? 16 : 4;
+        const bool skip = maybe && !rows;
+        cudaStream_t side = ctx->side_streams[0];
+        if (skip) {
+            // beside the tiles: a long pair's latency is theirs as a whole
+            cudaEventRecord(ctx->ev_fork, ctx->stream);
+            cudaStreamWaitEvent(side, ctx->ev_fork, 0);
+            a.shortest = 32 * (long_words(E_max) - 1) + 1;
+            st = ctx->cuda(launch_variant<PartitionedK>(a, ctx->sms, side),
+                           "pf_filter_partitioned launch");
+        }
+        const pf_status st2 = ctx->cuda(
+            launch_submat_sliced(filter_args_of(a), t, y, lanes, skip, ctx->sms, ctx->stream),
+            "pf_filter_partitioned launch");
+        if (skip) {
+            cudaEventRecord(ctx->ev_join[0], side);
+            cudaStreamWaitEvent(ctx->stream, ctx->ev_join[0], 0);
+        }
+        return st != PF_OK ? st : st2;
+    }
     return ctx->cuda(launch_variant<PartitionedK>(a, ctx->sms, ctx->stream),
                      "pf_filter_partitioned launch");
 }
