@@ -802,26 +802,35 @@ static int plain_index(int E_max) {
     return pi;
 }
 
-// How a batch below small_batch runs.  Measured (us) on 150 bp and on the mix of
-// 100/150/250 bp with thresholds of 0 to 10 % (E_max = 25), both deciders
-// unless said otherwise:
+// How a batch below small_batch runs.  The lines lie where the new side is not
+// slower for any of 100, 150 and 250 bp and their mix (us, 150 / 250 bp or the mix
+// of 100/150/250 bp with thresholds of 0 to E_max; a quarter accepted):
 //   wide    one warp per pair, the fused loop: the shortest latency.  Mix, plain
-//           -> wide: 1k pairs 65 -> 14, 16k 82 -> 37, 32k 96 -> 56 (bit-sliced 68);
-//           E_max = 15: 1k 27 -> 13, 16k 27 -> 32
+//           -> wide: E_max = 25 8k pairs 52 -> 25, 32k 96 -> 54 (both deciders);
+//           E_max = 15 8k 32 -> 22, 16k 34 -> 27 (100 and 150 bp alone 26 -> 26)
 //   sliced  grouped by threshold, then one bit-sliced launch with 16 lanes per
-//           group of 32 pairs (8 from 100k pairs of one threshold on).  Mix, plain ->
-//           sliced: 100k 265 -> 81, 1M 2609 -> 367; E_max = 15: 32k 29 -> 47,
-//           100k 74 -> 57; one threshold, 100k: E = 8 27 -> 29 (SneakySnake
-//           alone 29 -> 23), 10 36 -> 29, 12 46 -> 29, 25 (250 bp) 206 -> 56; 16k
-//           E = 12 21 -> 20; 50k E = 10 27 -> 23.  GateKeeper alone, mix: 100k 68 -> 68,
-//           200k 133 -> 88; up to E_max = 15 plain is as fast
-//   batched the scheduler with one bin: one threshold, 1M pairs, sliced ->
-//           batched: E = 8 173 -> 115, 12 172 -> 144; 400k 78 -> 83
+//           group of 32 pairs (8 from 100k pairs of one threshold on).
+//           Thresholds per pair, plain -> sliced: E_max = 25 50k 96 -> 70, 0.8M 984
+//           -> 279; E_max = 8..15, SneakySnake, whole path 100k 81 -> 82 (100 and
+//           150 bp), 150k 96 -> 103 / 107 -> 108, 200k 107 -> 103; both deciders
+//           75k 68 -> 84, 100k 82 -> 83, 300k 173 -> 129; GateKeeper, E_max = 25
+//           100k 49 -> 59, 150k 65 -> 71, 200k 92 -> 71 (up to 15 plain is as fast).
+//           One threshold: E = 8 SneakySnake 75k 20 -> 24 / 25 -> 33, 200k 42 -> 43 /
+//           55 -> 64, 0.3M 54 -> 45 / 71 -> 68, both 450k 79 -> 82 / 116 -> 127;
+//           E = 10 SneakySnake 50k 25 -> 23 / 31 -> 31, both 90k 32 -> 32 / 44 -> 46,
+//           150k 41 -> 32 / 54 -> 48; E = 12 both 35k 20 -> 23 / 25 -> 33, 40k 30 ->
+//           26 / 40 -> 38; E = 16 15k 39 -> 21 / 51 -> 30
+//   batched the scheduler with one bin, four lanes: one threshold, sliced ->
+//           batched: E = 10, both 450k 82 -> 101 / 127 -> 141, 600k 106 -> 108 / 169 ->
+//           174, 800k 147 -> 112 / 227 -> 180; plain -> batched: E = 7 both 450k 71
+//           -> 90 / 104 -> 140, 600k 92 -> 92 / 137 -> 148, 700k 103 -> 94 / 155 -> 152;
+//           SneakySnake 450k 68 -> 71 / 97 -> 115, 600k 87 -> 73 / 127 -> 123
 //   plain   one thread per pair, everything else
 int pf_ctx::small_route(unsigned dec, const FilterArgs &a) const {
     const bool gk = dec == 2;
     if (!a.E) {
-        if (a.n >= 450000 && !tune_plain[dec][a.E_max] &&
+        const int64_t batched_from = a.E_max > 8 ? 550000 : (dec == 1 ? 600000 : 650000);
+        if (a.n >= batched_from && !tune_plain[dec][a.E_max] &&
             cfg_sliced(kBatchCfgs[pf_default_cfg((int)dec, a.E_max)]))
             return kSmallBatched;
         if (a.E_max < (gk ? 16 : 8)) return kSmallPlain;
@@ -831,16 +840,17 @@ int pf_ctx::small_route(unsigned dec, const FilterArgs &a) const {
         // 16 lanes, 1.8 one by one (30,000 of 4,000 0.40 and 0.39)
         if (a.n < 40000 && long_rows(a, a.E_max) && row_words(a.pairs) >= 256) return kSmallBatched;
         const int64_t plain_below = a.E_max >= 16   ? 0
-                                    : a.E_max >= 12 ? 25000
-                                    : a.E_max >= 10 ? 50000
-                                    : dec == 1      ? 75000
+                                    : a.E_max >= 12 ? 40000
+                                    : a.E_max >= 10 ? (dec == 1 ? 50000 : 120000)
+                                    : dec == 1      ? 250000
+                                    : a.E_max == 8  ? batched_from
                                                     : 450000;
         if (a.n < plain_below) return kSmallPlain;
         return a.n < 100000 ? 16 : 8;
     }
     if (a.E_max < (gk ? 16 : 8)) return kSmallPlain;
     if (a.n <= (a.E_max >= 16 && !gk ? 40000 : 10000)) return kSmallWide;
-    if ((a.E_max < 16 && a.n < 75000) || (gk && a.n < 100000)) return kSmallPlain;
+    if ((a.E_max < 16 || gk) && a.n < (dec == 3 ? 100000 : 175000)) return kSmallPlain;
     return 16;
 }
 

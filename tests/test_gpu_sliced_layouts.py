@@ -85,7 +85,7 @@ def test_scheduler(pf, ctx, sides, per_pair):  # noqa: F811
 
 
 @pytest.mark.parametrize("sides", KINDS)
-@pytest.mark.parametrize("n,E,per_pair", [(30011, 13, False), (100031, 16, False),
+@pytest.mark.parametrize("n,E,per_pair", [(60011, 13, False), (100031, 16, False),
                                           (100031, 16, True), (1048700, 16, False)])
 def test_default_routes(pf, sides, n, E, per_pair):  # noqa: F811
     """16 lanes, 8 lanes, 16 lanes grouped, and the scheduler's default."""

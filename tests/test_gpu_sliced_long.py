@@ -42,7 +42,7 @@ def test_lengths_around_the_line(pf, ctx, E, share):  # noqa: F811
                           oracle.int_batch("ss_partitioned", P, p0=8, p1=2))
 
 
-@pytest.mark.parametrize("n,E", [(50_001, 13), (100_003, 9), (200_001, 20), (1_100_000, 10)])
+@pytest.mark.parametrize("n,E", [(50_001, 13), (300_003, 9), (200_001, 20), (1_100_000, 10)])
 @pytest.mark.parametrize("long", [0.01, 0.5])
 def test_default_routes(pf, n, E, long):  # noqa: F811
     """The routes at their default settings, over repeated pairs."""
