@@ -312,17 +312,17 @@ __device__ __forceinline__ void verify_two(const PairsView &pv, int64_t p, int64
         if (left > 8) b.eight<8>();
         if (left > 16) b.eight<16>();
         if (left > 24) b.eight<24>();
-        // as in verify_pair: out when both bands' smallest values are past
-        // their thresholds
+        // as in verify_pair: out when both pairs are over, by their bands'
+        // smallest values past the thresholds or by their ends (the columns
+        // behind a pair's end leave its distance as it is, so a short pair or an
+        // absent one does not hold a long one)
         const int ran = min((left + 7) & ~7, 32);
         T += ran - (int)((b.top & 0xffu) + ((b.top >> 8) & 0xffu));
         T2 += ran - (int)(((b.top >> 16) & 0xffu) + (b.top >> 24));
         b.top = 0u;
-        if (T - __popc(b.VN & 0xffffu) > E && T2 - __popc(b.VN >> 16) > E2) {
-            dist = E + 1;
-            dist2 = E2 + 1;
-            return;
-        }
+        if ((m - c <= 32 || T - __popc(b.VN & 0xffffu) > E) &&
+            (m2 - c <= 32 || T2 - __popc(b.VN >> 16) > E2))
+            break;
         a1 = a2;
         b1 = b2;
     }
