@@ -44,6 +44,9 @@ struct PairsView {
     SeqView read, ref;
 };
 
+// ceil(m / 32) for any length (m + 31 may not fit an int).
+__device__ __forceinline__ int words_of(int m) { return (int)(((unsigned)m + 31u) >> 5); }
+
 // One 32-bit word of each plane; words outside a sequence read as N.
 struct Word3 {
     uint32_t lo, hi, nm;

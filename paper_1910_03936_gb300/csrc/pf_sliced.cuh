@@ -210,7 +210,7 @@ struct SlicePairs {
         const int lane = threadIdx.x & 31;
         invalid = late = 0u;
         alone = false;
-        int lo = INT_MAX, hi = 0, wlo = INT_MAX, whi = 0;
+        int lo = INT_MAX, hi = 0;
         full = cnt == 32 * G;
 #pragma unroll
         for (int t = 0; t < G; ++t) {
@@ -233,11 +233,9 @@ struct SlicePairs {
         mmax = __reduce_max_sync(0xffffffffu, hi);
         const int most = 32 * (long_words(E) - 1);
         if (mmax > most) leave<FEW>(order, pos, cnt, E, most, to);
-        wlo = (mmin + 31) >> 5;
-        whi = (mmax + 31) >> 5;
         full = __all_sync(0xffffffffu, full);
         if (mmin > mmax) mmin = mmax;  // no valid pair
-        whole = full && wlo == whi;
+        whole = full && words_of(mmin) == words_of(mmax);
     }
 
     // The pairs of more than `most` columns leave the tile: into the list, or, in
@@ -284,12 +282,12 @@ struct SlicePairs {
     }
 
     // bit of every pair of the group that has a column i
-    __device__ __forceinline__ uint32_t valid(int i) const {
+    __device__ __forceinline__ uint32_t valid(unsigned i) const {
         const int lane = threadIdx.x & 31;
         const int q = lane / G;
         uint32_t v = 0u;
 #pragma unroll
-        for (int t = 0; t < G; ++t) v |= (m[t] > i ? 1u : 0u) << (t * L + q);
+        for (int t = 0; t < G; ++t) v |= ((unsigned)max(m[t], 0) > i ? 1u : 0u) << (t * L + q);
 #pragma unroll
         for (int o = G; o < 32; o <<= 1) v |= __shfl_xor_sync(0xffffffffu, v, o);
         return v;
@@ -327,7 +325,7 @@ struct SliceColumns {
         fx = rx + RC * G;
         rn = reinterpret_cast<uint32_t *>(fx + FC * G);
         fn = rn + RC * G;
-        W = (sp.mmax + 31) >> 5;
+        W = words_of(sp.mmax);
         even = true;
         if (!order && slice_strided(pv.read) && slice_strided(pv.ref)) {
             rbase = pos * pv.read.stride;
@@ -658,9 +656,10 @@ struct SliceWalk {
 
     // Whether columns from i on can change nothing: every pair that has them
     // (GateKeeper's counts lag `extra` columns) is past E by each decider.
-    __device__ __forceinline__ bool decided(const SlicePairs<L> &sp, int E, int i, int extra) const {
+    __device__ __forceinline__ bool decided(const SlicePairs<L> &sp, int E, unsigned i,
+                                            unsigned extra) const {
         uint32_t open = 0xffffffffu;
-        if (!sp.full || i - extra >= sp.mmin) open = sp.valid(i - extra);
+        if (!sp.full || i - extra >= (unsigned)sp.mmin) open = sp.valid(i - extra);
         if constexpr (SS)
             if (__any_sync(0xffffffffu, open & ~ss.above(E))) return false;
         if constexpr (GK) {
@@ -681,39 +680,43 @@ struct SliceWalk {
 // the warp's arrays at sm.
 template <int L, int DPT, typename Walk>
 __device__ __forceinline__ void slice_walk(const FilterArgs &a, const SlicePairs<L> &sp,
-                                           const int64_t *order, int64_t pos, int E, int extra,
+                                           const int64_t *order, int64_t pos, int E,
+                                           unsigned extra,
                                            uint32_t *sm, Walk &w) {
     using S = SliceShape<L, DPT>;
     constexpr int G = S::G, U = S::U, SEG = S::SEG;
     const int lane = threadIdx.x & 31;
-    const int total = sp.mmax + extra;
+    // (unsigned: columns past a length near INT_MAX)
+    const unsigned total = (unsigned)sp.mmax + extra;
+    const int words = (int)((total + 31u) >> 5);
     const bool one = sp.mmin == sp.mmax;
     SliceColumns<L> c;
     c.init(sm, a.pairs, sp, order, pos);
     w.clear();
     __syncwarp();
     c.vacant(-1);
-    for (int i0 = 0; i0 < total; i0 += 32 * SEG) {
-        c.load(a.pairs, sp, i0 >> 5);
-        if (i0 == 0) w.init(c, slice_first<L, DPT>(lane / G, E), E);
-        const int cols = min(32 * SEG, total - i0);
+    for (int w0 = 0; w0 < words; w0 += SEG) {
+        const unsigned i0 = 32u * (unsigned)w0;
+        c.load(a.pairs, sp, w0);
+        if (w0 == 0) w.init(c, slice_first<L, DPT>(lane / G, E), E);
+        const int cols = (int)min(32u * SEG, total - i0);
         for (int f = 0; f < cols; f += U) {
             uint32_t v[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) v[u] = 0xffffffffu;
-            if (i0 + f + U > sp.mmin) {
+            if (i0 + f + U > (unsigned)sp.mmin) {
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int i = i0 + f + u;
-                    v[u] = one ? (i < sp.mmax ? 0xffffffffu : 0u) : sp.valid(i);
+                    const unsigned i = i0 + f + u;
+                    v[u] = one ? (i < (unsigned)sp.mmax ? 0xffffffffu : 0u) : sp.valid(i);
                 }
             }
             w.block(c, f, v);
         }
         // (an obstacle of unrelated pairs comes every four columns or more; the
         // last words are not worth a vote)
-        const int i = i0 + 32 * SEG;
-        if (i >= 3 * E && total - i >= 64 && w.decided(sp, E, i, extra)) break;
+        const unsigned i = i0 + 32u * SEG;
+        if (i >= 3u * E && i + 64u <= total && w.decided(sp, E, i, extra)) break;
     }
 }
 

@@ -257,10 +257,11 @@ struct TwoBands {
     }
 };
 
-// Word w of a pair's planes, 0 (no N) behind its length.
-__device__ __forceinline__ Word3 load_ended(const SeqView &s, int64_t start, int w, int W, int m) {
+// Word w of a pair's planes, 0 (no N) behind the `rest` columns from there on.
+__device__ __forceinline__ Word3 load_ended(const SeqView &s, int64_t start, int w, int W,
+                                            int rest) {
     Word3 x = load_word(s, start, w, W);
-    const uint32_t past = __funnelshift_lc(0u, 0xffffffffu, (unsigned)max(m - 32 * w, 0));
+    const uint32_t past = __funnelshift_lc(0u, 0xffffffffu, (unsigned)max(rest, 0));
     x.lo &= ~past;
     x.hi &= ~past;
     x.nm &= ~past;
@@ -270,8 +271,7 @@ __device__ __forceinline__ Word3 load_ended(const SeqView &s, int64_t start, int
 // Distances of pairs p and p2 (lengths m and m2 >= 0, thresholds at most kTwoE).
 __device__ __forceinline__ void verify_two(const PairsView &pv, int64_t p, int64_t p2, int m,
                                            int m2, int E, int E2, int &dist, int &dist2) {
-    const int W = (m + 31) >> 5, W2 = (m2 + 31) >> 5;
-    const int longer = max(m, m2);
+    const int W = words_of(m), W2 = words_of(m2);
     const int64_t ra = pv.read.start(p), rb = pv.read.start(p2);
     const int64_t fa = pv.ref.start(p), fb = pv.ref.start(p2);
     TwoBands b;
@@ -287,10 +287,13 @@ __device__ __forceinline__ void verify_two(const PairsView &pv, int64_t p, int64
     b.hi.z[3] = low(a1.hi, b1.hi);
     b.nm.z[3] = low(a1.nm, b1.nm);
     int T = kTwoE, T2 = kTwoE;
-    for (int c = 0, fw = 0; c < longer; c += 32, ++fw) {
-        const Word3 f = load_ended(pv.ref, fa, fw, W, m), g = load_ended(pv.ref, fb, fw, W2, m2);
-        const Word3 a2 = load_ended(pv.read, ra, fw + 1, W, m);
-        const Word3 b2 = load_ended(pv.read, rb, fw + 1, W2, m2);
+    const int words = max(W, W2);
+    for (int fw = 0; fw < words; ++fw) {
+        const int rest = m - 32 * fw, rest2 = m2 - 32 * fw;
+        const Word3 f = load_ended(pv.ref, fa, fw, W, rest);
+        const Word3 g = load_ended(pv.ref, fb, fw, W2, rest2);
+        const Word3 a2 = load_ended(pv.read, ra, fw + 1, W, rest - 32);
+        const Word3 b2 = load_ended(pv.read, rb, fw + 1, W2, rest2 - 32);
         auto roll = [&](TwoPlanes &x, uint32_t a_now, uint32_t b_now, uint32_t a_next,
                         uint32_t b_next) {
             x.z[0] = x.z[2];
@@ -307,7 +310,7 @@ __device__ __forceinline__ void verify_two(const PairsView &pv, int64_t p, int64
         b.fhi[1] = high(f.hi, g.hi);
         b.fnm[0] = low(f.nm, g.nm);
         b.fnm[1] = high(f.nm, g.nm);
-        const int left = longer - c;
+        const int left = min(max(rest, rest2), 32);
         b.eight<0>();
         if (left > 8) b.eight<8>();
         if (left > 16) b.eight<16>();
@@ -316,12 +319,12 @@ __device__ __forceinline__ void verify_two(const PairsView &pv, int64_t p, int64
         // smallest values past the thresholds or by their ends (the columns
         // behind a pair's end leave its distance as it is, so a short pair or an
         // absent one does not hold a long one)
-        const int ran = min((left + 7) & ~7, 32);
+        const int ran = (left + 7) & ~7;
         T += ran - (int)((b.top & 0xffu) + ((b.top >> 8) & 0xffu));
         T2 += ran - (int)(((b.top >> 16) & 0xffu) + (b.top >> 24));
         b.top = 0u;
-        if ((m - c <= 32 || T - __popc(b.VN & 0xffffu) > E) &&
-            (m2 - c <= 32 || T2 - __popc(b.VN >> 16) > E2))
+        if ((rest <= 32 || T - __popc(b.VN & 0xffffu) > E) &&
+            (rest2 <= 32 || T2 - __popc(b.VN >> 16) > E2))
             break;
         a1 = a2;
         b1 = b2;

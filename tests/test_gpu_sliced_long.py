@@ -144,3 +144,38 @@ def test_long_pairs_take_no_longer_than_by_the_word_kernels(pf, spikes):  # noqa
         assert int(cnt.abs().sum()) == 0 and bool((acc == 1).all())
     finally:
         pf.pf_destroy(c)
+
+
+def test_lengths_near_the_largest_int(pf):  # noqa: F811
+    """Unrelated pairs of up to 2^31 - 1 bases (all share one read and one
+    reference): column counts past the length do not fit an int."""
+    top, n, E = 2**31 - 1, 100_010, 20
+    g = torch.Generator(device=DEV)
+    g.manual_seed(2)
+    word = lambda: torch.randint(-2**31, 2**31 - 1, (1 << 26,), generator=g,
+                                 device=DEV).to(torch.int32)
+    nm = torch.zeros(1 << 26, dtype=torch.int32, device=DEV)
+    off = torch.zeros(n, dtype=torch.int64, device=DEV)
+    pairs = pf.Pairs(pf.Seqs(word(), word(), nm, word_off=off), pf.Seqs(word(), word(), nm, word_off=off))
+    lens = (top - torch.arange(n, device=DEV) % 40).to(torch.int32)
+    lens[5::64] = 100
+    Ed = torch.full((n,), E, dtype=torch.int16, device=DEV)
+    Ed[::3] = 17
+    new = lambda: (torch.full((2 * n,), 9, dtype=torch.uint8, device=DEV),
+                   torch.full((2 * n,), 99, dtype=torch.int16, device=DEV))
+    c = pf.pf_create(0)
+    try:
+        for e in (None, Ed):
+            for dec in (1, 2, 3):
+                got, want = new(), new()
+                pf.pf_filter(c, dec, pairs, lens, e, E, *got, n)
+                pf.pf_filter_plain(c, dec, pairs, lens, e, E, *want, n)
+                pf.pf_sync(c)
+                assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+                assert not got[0][:n][lens > 100].any()
+        dist = torch.full((n,), -7, dtype=torch.int32, device=DEV)
+        pf.pf_verify(c, pairs, lens, None, 6, None, None, dist, n)   # two pairs to a word
+        pf.pf_sync(c)
+        assert bool((dist == 7).all())
+    finally:
+        pf.pf_destroy(c)
