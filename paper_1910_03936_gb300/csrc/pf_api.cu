@@ -519,10 +519,18 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
         if (next++ < kSideStreams) cudaStreamWaitEvent(x, ev_fork, 0);
         return x;
     };
+    // every way out from here on: the side streams' work before ours
+    auto join = [&]() {
+        for (int i = 0; i < kSideStreams && i < next; ++i) {
+            cudaEventRecord(ev_join[i], side_streams[i]);
+            cudaStreamWaitEvent(stream, ev_join[i], 0);
+        }
+        return st;
+    };
     b.want = 1;
     if (wide.count) {
         st = cuda(launch_filter_slices((int)dec, 16, b, wide, -1, sms, side()), "filter launch");
-        if (st != PF_OK) return st;
+        if (st != PF_OK) return join();
     }
     b.want = 0;
     if (few)
@@ -544,7 +552,7 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
             if (!bins.count) continue;
             st = cuda(launch_filter_slice_bins((int)dec, cls, b, bins, sms, side()),
                       "filter launch");
-            if (st != PF_OK) return st;
+            if (st != PF_OK) return join();
         }
     }
     for (const int c : used) {
@@ -555,7 +563,7 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
             if (tune_cfg[dec][e] == c) bi.chunk = tune_chunk[dec][e];
         const int grid = grid_for(dec, c);
         st = cuda(launch_filter_batched(dec, c, grid, bi, c, side()), "filter launch");
-        if (st != PF_OK) return st;
+        if (st != PF_OK) return join();
     }
     b.want = 1;
     for (int i = 0; i < sliced.count && sliced.E[i] <= kWordsTo; ++i) {
@@ -564,12 +572,9 @@ pf_status pf_ctx::run_batched(unsigned dec, const FilterArgs &a, const Scratch &
         const int c = pf_long_cfg(sliced.E[i], false);
         st = cuda(launch_filter_batched(dec, c, grid_for(dec, c), bi, sliced.bin[i], side()),
                   "filter launch");
-        if (st != PF_OK) return st;
+        if (st != PF_OK) return join();
     }
-    for (int i = 0; i < kSideStreams && i < next; ++i) {
-        cudaEventRecord(ev_join[i], side_streams[i]);
-        cudaStreamWaitEvent(stream, ev_join[i], 0);
-    }
+    join();
     st = cuda(cudaGetLastError(), "filter launch");
     return st == PF_OK && list ? run_late(dec, a, s) : st;
 }
