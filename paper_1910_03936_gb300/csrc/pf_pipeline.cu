@@ -10,9 +10,9 @@
 // with more, full chunks replay a graph captured once per slot.
 //
 // The call is bound by the upload; what it adds is what comes before the first
-// copy and after the last.  So a slot is set up only when its first chunk comes
-// (the second under the first's upload), and its memory and stream stay with
-// the context.  1.5M pairs of 150 bp in two chunks: 3320 us with four graphs
+// copy and after the last.  So a slot's memory and stream stay with the context.
+// (Both are there before the first upload: a call that cannot get them has
+// written nothing.)  1.5M pairs of 150 bp in two chunks: 3320 us with four graphs
 // captured and both slots allocated and freed by every call, 2380 us now (the
 // upload of 450 MB 2130).
 #include <algorithm>
@@ -291,16 +291,12 @@ extern "C" pf_status pf_run_host(pf_ctx *ctx, unsigned deciders, const uint8_t *
         if (c >= 0) ctx->grid_for((int)deciders, c);
     }
     const bool replay = n / J.C >= kGraphChunks;
-    for (int i = 0; i < 2 && replay && st == PF_OK; ++i) {
+    for (int i = 0; i < 2 && i < nchunks && st == PF_OK; ++i) {
         st = setup_slot(J, slots[i], i);
-        if (st == PF_OK) st = capture(J, slots[i], J.C, &slots[i].exec);
+        if (st == PF_OK && replay) st = capture(J, slots[i], J.C, &slots[i].exec);
     }
     for (int64_t c = 0; c < nchunks && st == PF_OK; ++c) {
         Slot &s = slots[c & 1];
-        if (!s.st) {
-            st = setup_slot(J, s, (int)(c & 1));
-            if (st != PF_OK) break;
-        }
         const int64_t c0 = c * J.C, nc = std::min(J.C, n - c0);
         // the slot's previous chunk: results are in host memory once its
         // copies (queued on the same stream) are done
