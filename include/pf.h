@@ -444,7 +444,8 @@ PF_API pf_status pf_host_free(void *ptr);
  * Page-locked host buffers (pf_host_alloc's, or any registered memory)
  * are copied asynchronously; pageable ones work but serialise the copies.
  * Allocates its slot buffers; they stay with the context for later calls up to
- * 1 GiB a slot (larger ones are freed on return) and are freed by pf_destroy. */
+ * 1 GiB a slot (larger ones are freed on return) and are freed by pf_destroy,
+ * or by a later call on the context that finds no memory otherwise. */
 PF_API pf_status pf_run_host(pf_ctx *ctx, unsigned deciders, const uint8_t *reads,
                              const uint8_t *refs, const int64_t *byte_off, int len,
                              const int16_t *E, int E_max, uint8_t *accept, int16_t *count,

@@ -244,6 +244,25 @@ pf_status pf_ctx::cuda(cudaError_t e, const char *what) {
     return fail(PF_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+bool pf_ctx::alloc(void **p, size_t bytes) {
+    *p = nullptr;
+    if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+    cudaGetLastError();
+    *p = nullptr;
+    bool kept = false;
+    for (HostSlot &h : host_slots) {
+        if (!h.mem) continue;
+        cudaFree(h.mem);
+        h.mem = nullptr;
+        h.bytes = 0;
+        kept = true;
+    }
+    if (kept && cudaMalloc(p, bytes) == cudaSuccess) return true;
+    cudaGetLastError();
+    *p = nullptr;
+    return false;
+}
+
 pf_status pf_ctx::ensure_scratch(size_t bytes) {
     if (bytes <= scratch_bytes) return PF_OK;
     verified_state = 0;
@@ -256,11 +275,8 @@ pf_status pf_ctx::ensure_scratch(size_t bytes) {
     size_t want = std::max(bytes, scratch_bytes * 3 / 2);
     if (cudaMalloc(&scratch, want) != cudaSuccess) {
         cudaGetLastError();
-        if (cudaMalloc(&scratch, bytes) != cudaSuccess) {
-            cudaGetLastError();
-            scratch = nullptr;
+        if (!alloc(&scratch, bytes))
             return fail(PF_ENOMEM, "scratch allocation of %zu bytes failed", bytes);
-        }
         want = bytes;
     }
     scratch_bytes = want;
@@ -1089,12 +1105,11 @@ pf_status pf_tune_batch(pf_ctx *ctx, unsigned deciders, const pf_pairs *pairs,
     int16_t *cnt = nullptr;
     int64_t *range = nullptr;  // [2] positions timed, then the work counter
     int64_t *sample_order = nullptr;
-    if (cudaMalloc(&acc, (size_t)slots * n) != cudaSuccess ||
-        cudaMalloc(&cnt, (size_t)slots * n * sizeof(int16_t)) != cudaSuccess ||
-        cudaMalloc(&range, 4 * sizeof(int64_t)) != cudaSuccess ||
-        cudaMalloc(&sample_order, (size_t)std::min<int64_t>(sample, n) * sizeof(int64_t)) !=
-            cudaSuccess) {
-        cudaGetLastError();
+    if (!ctx->alloc((void **)&acc, (size_t)slots * n) ||
+        !ctx->alloc((void **)&cnt, (size_t)slots * n * sizeof(int16_t)) ||
+        !ctx->alloc((void **)&range, 4 * sizeof(int64_t)) ||
+        !ctx->alloc((void **)&sample_order,
+                    (size_t)std::min<int64_t>(sample, n) * sizeof(int64_t))) {
         if (acc) cudaFree(acc);
         if (cnt) cudaFree(cnt);
         if (range) cudaFree(range);
@@ -1232,9 +1247,8 @@ pf_status pf_tune(pf_ctx *ctx, unsigned deciders, const pf_pairs *pairs, const i
     uint8_t *acc = nullptr;
     int16_t *cnt = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (cudaMalloc(&acc, (size_t)slots * n) != cudaSuccess ||
-        cudaMalloc(&cnt, (size_t)slots * n * sizeof(int16_t)) != cudaSuccess) {
-        cudaGetLastError();
+    if (!ctx->alloc((void **)&acc, (size_t)slots * n) ||
+        !ctx->alloc((void **)&cnt, (size_t)slots * n * sizeof(int16_t))) {
         if (acc) cudaFree(acc);
         return ctx->fail(PF_ENOMEM, "pf_tune: output buffers");
     }

@@ -83,6 +83,8 @@ struct pf_ctx {
 
     pf_status fail(pf_status s, const char *fmt, ...);
     pf_status cuda(cudaError_t e, const char *what);
+    // device memory, if need be in place of what pf_run_host keeps
+    bool alloc(void **p, size_t bytes);
     pf_status ensure_scratch(size_t bytes);
     pf_status scratch_layout(int64_t n, pf::Scratch *s);
     int grid_for(int dec, int cfg);

@@ -581,7 +581,7 @@ pf_status pf_serve_start(pf_ctx *ctx, const pf_serve_config *cfg) {
         S->th = std::thread(batch_scheduler, S);
         return PF_OK;
     }
-    bool ok = cudaMalloc(&S->arena, budget) == cudaSuccess &&
+    bool ok = ctx->alloc((void **)&S->arena, budget) &&
               cudaMalloc(&S->d_desc, sizeof(ServeDesc) * c.max_requests) == cudaSuccess &&
               cudaMalloc(&S->d_done, sizeof(unsigned) * c.max_requests) == cudaSuccess &&
               cudaMalloc(&S->d_head, sizeof(unsigned long long)) == cudaSuccess &&

@@ -508,8 +508,7 @@ pf_status batch_start(pf_ctx *ctx, ServeState *Sp) {
         o_ro[i] = add((nn + kMaxSegs) * 8);
         o_re[i] = add(nn * 2);
     }
-    if (cudaMalloc(&B.mem, o) != cudaSuccess) {
-        cudaGetLastError();
+    if (!ctx->alloc((void **)&B.mem, o)) {
         return ctx->fail(PF_ENOMEM, "serve batch buffers (%zu bytes)", o);
     }
     char *m = B.mem;

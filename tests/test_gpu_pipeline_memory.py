@@ -58,3 +58,44 @@ def test_a_call_without_room_for_both_slots_writes_nothing(pf):
         assert (out[0] == 1).all() and not out[1].any() and not out[2].any()
     finally:
         pf.pf_destroy(c)
+
+
+@pytest.mark.parametrize("what", ["filter", "tune", "serve", "serve loop"])
+def test_kept_slots_make_room_for_other_calls(pf, what):
+    """What pf_run_host keeps (two slots of 0.9 GB) is given back where another
+    call of the context needs the memory."""
+    m, chunk = 8_000, 37_000
+    reads = pair_bytes(2 * chunk, m)
+    n = {"filter": 45_000_000, "tune": 60_000_000}.get(what, 1)
+    lens = torch.full((n,), 32, dtype=torch.int32, device=DEV)
+    word = torch.zeros(1, dtype=torch.int32, device=DEV)
+    pairs = pf.Pairs(pf.Seqs(word, word, word), pf.Seqs(word, word, word))   # all the same
+    acc = torch.zeros(n if what == "filter" else 1, dtype=torch.uint8, device=DEV)
+    cnt = torch.zeros(n if what == "filter" else 1, dtype=torch.int16, device=DEV)
+    c = pf.pf_create(0)
+    try:
+        if what == "tune":   # scratch for n pairs is there, the tuner's outputs are not
+            a, k = (torch.zeros(n, dtype=t, device=DEV) for t in (torch.uint8, torch.int16))
+            pf.pf_filter(c, 1, pairs, lens, None, 0, a, k, n)
+            pf.pf_sync(c)
+            del a, k
+        pf.pf_run_host(c, 1, reads, reads, 2, length=m, chunk_pairs=chunk)
+        room = 130_000_000 if what == "tune" else 600_000_000
+        held = leave_free(room)
+        try:
+            assert torch.cuda.mem_get_info()[0] < room + 40_000_000
+            if what == "filter":
+                pf.pf_filter(c, 1, pairs, lens, None, 0, acc, cnt, n)
+                pf.pf_sync(c)
+                assert bool((acc == 1).all()) and not bool(cnt.any())
+            elif what == "tune":
+                pf.pf_tune(c, 1, pairs, lens, 0, reps=1)
+            else:
+                mode = {"mode": 1} if what == "serve loop" else {}
+                pf.pf_serve_start(c, hbm_budget=900_000_000, **mode)
+                pf.pf_serve_stop(c)
+        finally:
+            held.clear()
+            torch.cuda.empty_cache()
+    finally:
+        pf.pf_destroy(c)
