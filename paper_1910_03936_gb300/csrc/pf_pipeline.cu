@@ -287,9 +287,11 @@ extern "C" pf_status pf_run_host(pf_ctx *ctx, unsigned deciders, const uint8_t *
     // occupancy queries (the first of a kernel loads it) and captures before the
     // first upload
     for (int e = E ? 0 : E_max; e <= E_max; ++e) {
-        const int c = ctx->tune_cfg[deciders][e];
-        if (c >= 0) ctx->grid_for((int)deciders, c);
+        ctx->grid_for((int)deciders, ctx->tune_cfg[deciders][e]);
+        ctx->grid_for((int)deciders, pf_long_cfg(e, false));
     }
+    ctx->grid_for((int)deciders, kWideCfg);
+    ctx->grid_for((int)deciders, pf_long_cfg(E_max, true));
     const bool replay = n / J.C >= kGraphChunks;
     for (int i = 0; i < 2 && i < nchunks && st == PF_OK; ++i) {
         st = setup_slot(J, slots[i], i);
