@@ -205,8 +205,13 @@ static cudaError_t launch_binning(const FilterArgs &a, const BinTable &t, int nb
 }
 
 // Whether the pairs that a bin runs together lie together: *scattered = 0 when
-// most of 1,024 sampled neighbours in the bins' order are neighbours in the
-// read's planes (the layout grouped by threshold and length), else 1.
+// 200 of 1,024 sampled neighbours in the bins' order are neighbours in the read's
+// planes (the layout grouped by threshold and length), else 1.  The scatter mixes
+// a bin's pairs within a tile, so that even a sorted batch has about 460.  3M
+// pairs of k thresholds, SneakySnake, four lanes / 16, ms: grouped k = 9 (670) 0.56
+// / 0.81, k = 26 and three lengths (330) 0.70 / 0.76; pair order k = 2 (280) 0.61 /
+// 0.84, k = 4 (180) 0.86 / 0.85, k = 2 and three lengths (140) 1.31 / 0.96, k = 9
+// (100) 1.26 / 0.90.
 __global__ void __launch_bounds__(1024)
 bin_layout_kernel(SeqView read, const int32_t *lens, const int64_t *order, const int *ident,
                   int64_t n, int *scattered) {
@@ -215,7 +220,7 @@ bin_layout_kernel(SeqView read, const int32_t *lens, const int64_t *order, const
     const int64_t p = id ? q : order[q], p2 = id ? q + 1 : order[q + 1];
     const bool near = read.start(p2) - read.start(p) == (int64_t)((lens[p] + 31) >> 5);
     const int c = __syncthreads_count(near);
-    if (threadIdx.x == 0) *scattered = c < 512;
+    if (threadIdx.x == 0) *scattered = c < 200;
 }
 
 }  // namespace pf
