@@ -189,6 +189,12 @@ PF_API pf_status pf_pack_fixed(pf_ctx *ctx, const uint8_t *ascii, int64_t nseq, 
  * pairs are grouped by the configuration their threshold is tuned to and,
  * inside a group, by length class (ceil(len/32) words); each group runs the
  * tuned mapping (threads per pair, work chunk) in one persistent launch.
+ * Bit-sliced configurations (pf_kernel_configs) are taken as a choice of the
+ * method: with thresholds of their own, short groups share a launch; batches
+ * below 1.6M pairs, and those whose groups' pairs are scattered over the planes
+ * (pair order), run them with 16 lanes per 32 pairs, and up to E = 10 with one
+ * thread per pair; pairs of 12 words and more (16 from E = 10 on, 21 from E = 16
+ * on) run one by one.  Results are the same.
  * Batches below pf_set_small_batch's size take one launch: the plain kernel
  * (with one threshold for the batch, E NULL and E_max <= 15, fixed at
  * compile time), one warp per pair, or, after grouping the pairs by
@@ -269,8 +275,9 @@ PF_API pf_status pf_set_resolve_by_bounds(pf_ctx *ctx, int enable);
  * -1 selects the plain kernel.  PF_EINVAL if cfg cannot serve E. */
 PF_API pf_status pf_tune_set(pf_ctx *ctx, unsigned deciders, int E, int cfg, int chunk);
 
-/* The configuration and chunk currently used for (deciders, E); cfg = -1
- * when pf_tune chose the plain kernel. */
+/* The configuration and chunk currently chosen for (deciders, E) (pf_filter says
+ * where a bit-sliced one runs in another form); cfg = -1 when pf_tune chose the
+ * plain kernel. */
 PF_API pf_status pf_tune_get(pf_ctx *ctx, unsigned deciders, int E, int *cfg, int *chunk);
 
 /* Autotuner: time every configuration that serves E, with work chunks of

@@ -319,6 +319,8 @@ pf_status pf_ctx::scratch_layout(int64_t n, Scratch *s) {
     return PF_OK;
 }
 
+// Blocks of a persistent launch.  (Bit-sliced launches with tables of starts hold
+// up to 4 KB more shared memory per block than asked for here; 12 still fit.)
 int pf_ctx::grid_for(int dec, int cfg) {
     int &g = grid_cache[dec][cfg];
     if (g == 0) {

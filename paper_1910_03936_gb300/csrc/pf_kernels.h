@@ -104,8 +104,8 @@ inline int64_t row_words(const PairsView &pv) {
     return r.off || f.off || lo < 1 ? INT64_MAX : (r.stride > f.stride ? r.stride : f.stride);
 }
 // Warps per SM that a kernel's registers are held to.  More warps hide more
-// latency but leave less L1 for the loads (the walk's arrays take 13.6 KB per
-// warp).  SneakySnake, 12 / 9 warps: 0.285 / 0.283 ms for 4M pairs of 150 bp at
+// latency but leave less L1 for the loads (the walk's arrays take 12.6 KB per
+// warp, 14.6 or 16.6 with the tables of starts).  SneakySnake, 12 / 9 warps: 0.285 / 0.283 ms for 4M pairs of 150 bp at
 // E = 6, 0.332 / 0.327 at E = 15, 0.382 / 0.366 for 2M of 250 bp at E = 25; with
 // GateKeeper, which keeps four columns of every diagonal: E = 6 12 / 9 warps
 // 0.353 / 0.359, E = 15 9 / 8 warps 0.503 / 0.535, E = 25 9 (spills) / 8 warps

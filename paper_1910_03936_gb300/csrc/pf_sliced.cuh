@@ -8,9 +8,9 @@
 // (no shift), every decider is a fixed sequence of logic operations per column
 // (no divergence), and a count is a few bit planes (a vertical counter).
 // Per column, diagonal and 32 pairs: two logic operations for the mismatch
-// cell (three with the reference's N folded in, which GateKeeper needs), one
-// and a half for SneakySnake, three for GateKeeper, against about 13 and
-// 10 + a share of the step loop in the word-per-pair form.
+// cell (three with the reference's N folded in, which GateKeeper needs), two
+// for SneakySnake, three for GateKeeper, against about 13 and 10 + a share of
+// the step loop in the word-per-pair form.
 //
 // One warp takes a tile of G = 32 / L groups; the L lanes of a group share
 // its 32 pairs and split the 2E + 1 diagonals, DPT consecutive ones per lane

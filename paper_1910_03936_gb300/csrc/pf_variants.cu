@@ -548,7 +548,7 @@ extern "C" pf_status pf_filter_partitioned(pf_ctx *ctx, const pf_pairs *pairs,
     cudaSetDevice(ctx->device);
     VariantArgs a = variant_args_of(ctx, pairs, lens, E, E_max, t, y, accept, count, n);
     // One threshold: bit-sliced tiles, whose time does not depend on t and y.
-    // One pair per lane group costs about (E + 2) * steps, steps = 32 y / t per
+    // One pair a thread costs about (E + 2) * steps, steps = 32 y / t per
     // word.  2M pairs of 150 bp, E = 6, t = 8, y = 2 (64): 395 us so, 183 in
     // tiles; t = 32, y = 1 (8): 177 and 182; 250 bp, E = 25, t = 8, y = 2:
     // 2810 and 441.  Few pairs leave tiles without enough warps: 100,000 of the
