@@ -1036,14 +1036,15 @@ def main_gpu(args):
     # kernels of ours launched per step: 2 pack, binning (init, and with
     # several configurations histogram, scan, scatter), one filter launch per
     # distinct configuration serving E = 0..E_HEAD (a per-pair E array can
-    # hold any of them), 3 compaction, 1 verification; with a bit-sliced one
-    # among several also the check of the pairs' order and the launch for
-    # scattered pairs
+    # hold any of them), 3 compaction, 1 verification; with bit-sliced ones
+    # among several also the check of the pairs' order and for each the exact
+    # kernel that scattered pairs take (up to E = 10)
     chosen = {pf.pf_tune_get(ctx, 3, e)[0] for e in range(E_HEAD + 1)}
     n_cfg = len(chosen)
     table = pf.pf_kernel_configs()
-    sliced = any(c >= 0 and table[c][3] >= 0 and table[c][0] > 1 for c in chosen)
-    line["gpu_launches"] = args.steps * (2 + (1 if n_cfg == 1 else 4 + 2 * sliced) + n_cfg + 3 + 1)
+    sliced = sum(c >= 0 and table[c][3] >= 0 and table[c][0] > 1 for c in chosen)
+    order = 1 + sliced if sliced else 0
+    line["gpu_launches"] = args.steps * (2 + (1 if n_cfg == 1 else 4 + order) + n_cfg + 3 + 1)
     if rank == 0 and world == 1 and not args.no_cpu:
         r, dt, thr = oracle_step_rate(args.cpu_sample)
         r1, dt1, _ = oracle_step_rate(args.cpu_sample_1t, threads=1)
