@@ -381,7 +381,7 @@ static bool long_rows(const FilterArgs &a, int E) {
 }
 
 static LongPairs list_of(const Scratch &s) {
-    return {true, s.idx, reinterpret_cast<unsigned long long *>(s.late() + 1)};
+    return {true, false, s.idx, reinterpret_cast<unsigned long long *>(s.late() + 1)};
 }
 
 // E = 0 compares one diagonal and is bound by memory: the plain kernel
@@ -840,9 +840,10 @@ static int plain_index(int E_max) {
 //           group of 32 pairs (8 from 100k pairs of one threshold on).
 //           Thresholds per pair, plain -> sliced: E_max = 25 50k 96 -> 70, 0.8M 984
 //           -> 279; E_max = 8..15, SneakySnake, whole path 100k 81 -> 82 (100 and
-//           150 bp), 150k 96 -> 103 / 107 -> 108, 200k 107 -> 103; both deciders
-//           75k 68 -> 84, 100k 82 -> 83, 300k 173 -> 129; GateKeeper, E_max = 25
-//           100k 49 -> 59, 150k 65 -> 71, 200k 92 -> 71 (up to 15 plain is as fast).
+//           150 bp; E_max = 15 the filter alone 58 -> 52), 150k 96 -> 103 / 107 -> 108,
+//           200k 107 -> 103; both deciders 75k 68 -> 84, 100k 82 -> 83, 300k 173 ->
+//           129; GateKeeper, E_max = 25 100k 49 -> 59, 150k 65 -> 71, 200k 92 -> 71
+//           (up to 15 plain is as fast).
 //           One threshold: E = 8 SneakySnake 75k 20 -> 24 / 25 -> 33, 200k 42 -> 43 /
 //           55 -> 64, 0.3M 54 -> 45 / 71 -> 68, both 450k 79 -> 82 / 116 -> 127;
 //           E = 10 SneakySnake 50k 25 -> 23 / 31 -> 31, both 90k 32 -> 32 / 44 -> 46,
@@ -878,7 +879,8 @@ int pf_ctx::small_route(unsigned dec, const FilterArgs &a) const {
     }
     if (a.E_max < (gk ? 16 : 8)) return kSmallPlain;
     if (a.n <= (a.E_max >= 16 && !gk ? 40000 : 10000)) return kSmallWide;
-    if ((a.E_max < 16 || gk) && a.n < (dec == 3 ? 100000 : 175000)) return kSmallPlain;
+    if ((a.E_max < 16 || gk) && a.n < (dec == 3 || (a.E_max == 15 && !gk) ? 100000 : 175000))
+        return kSmallPlain;
     return 16;
 }
 

@@ -105,10 +105,11 @@ struct FilterArgs {
 // at E = 20 640 bp 1.84 / 3.08, 1000 bp 3.26 / 1.85 (1M pairs).
 __host__ __device__ constexpr int long_words(int E) { return E < 10 ? 12 : (E < 16 ? 16 : 21); }
 
-// Where a tile leaves its long pairs (off: it walks them).
+// Where a tile leaves its long pairs (off: it walks them; few: unless they are
+// more than an eighth of its pairs).
 struct LongPairs {
-    bool on = false;
-    int64_t *list = nullptr;                // null: another launch finds them by their lengths
+    bool on = false, few = false;
+    int64_t *list = nullptr;                // null: another launch finds them
     unsigned long long *count = nullptr;    // zeroed
 };
 

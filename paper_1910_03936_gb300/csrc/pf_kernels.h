@@ -190,9 +190,11 @@ cudaError_t launch_filter_slices(int dec, int lanes, const BatchArgs &b, const S
                                  int single, int sms, cudaStream_t st);
 
 // SneakySnake on sub-matrices (t columns, y replications), one threshold, 16 or
-// four lanes per group; skip_long: long pairs are left out.
-cudaError_t launch_submat_sliced(const FilterArgs &a, int t, int y, int lanes, bool skip_long,
-                                 int sms, cudaStream_t st);
+// four lanes per group; late: which long pairs are left out (with few, their
+// counts are kLeftOut then).
+constexpr int16_t kLeftOut = -2;
+cudaError_t launch_submat_sliced(const FilterArgs &a, int t, int y, int lanes,
+                                 const LongPairs &late, int sms, cudaStream_t st);
 
 cudaError_t launch_pack_ragged(const uint8_t *ascii, const int64_t *byte_off,
                                const int64_t *word_off, int64_t nseq, uint32_t *lo,

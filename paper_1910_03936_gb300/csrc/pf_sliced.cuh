@@ -247,15 +247,19 @@ struct SlicePairs {
     __device__ __forceinline__ void leave(const int64_t *order, int64_t pos, int cnt, int E,
                                           int most, const LongPairs &to) {
         const int lane = threadIdx.x & 31;
-        bool list = to.list != nullptr;
-        if constexpr (FEW) {
+        bool list = to.list != nullptr, some = true;
+        if (!FEW && !to.on) return;
+        if (FEW || to.few) {
             int n = 0;
 #pragma unroll
             for (int t = 0; t < G; ++t) n += __popc(__ballot_sync(0xffffffffu, m[t] > most));
-            alone = 8 * n <= cnt;
+            some = 8 * n <= cnt;
+        }
+        if constexpr (FEW) {
+            alone = some;
             if (!alone && (E >= 16 || !list)) return;
             if (alone) list = false;
-        } else if (!to.on) {
+        } else if (!some) {
             return;
         }
         int lo = INT_MAX, hi = 0;
@@ -778,8 +782,12 @@ submat_sliced_kernel(FilterArgs a, int t, int y, LongPairs late) {
         slice_walk<L, DPT>(a, sp, nullptr, pos, E, 0, slice_sm, w);
 #pragma unroll
         for (int k = 0; k < S::G; ++k) {
-            if (32 * k + lane >= cnt || ((sp.late >> k) & 1u)) continue;
+            if (32 * k + lane >= cnt) continue;
             const int64_t p = pos + 32 * k + lane;
+            if ((sp.late >> k) & 1u) {
+                if (late.few) a.count[p] = kLeftOut;
+                continue;
+            }
             if ((sp.invalid >> k) & 1u) write_invalid<1>(a, p);
             else write_outputs<1>(a, p, E, w.ss.get(k * L + lane / S::G, E + 1), 0, 0);
         }

@@ -24,7 +24,10 @@ struct VariantArgs {
     const int16_t *E;  // null: E_max for every pair
     int E_max;
     int p0, p1;        // t and y, or the SHD flags
-    int shortest = 0;  // partitioned_kernel: pairs of fewer columns are left out
+    // partitioned_kernel: pairs of fewer columns are left out, or all but those
+    // whose count is kLeftOut
+    int shortest = 0;
+    bool left_out = false;
     uint8_t *accept;
     int16_t *count;
     int64_t n;
@@ -110,6 +113,7 @@ __global__ void __launch_bounds__(256) partitioned_kernel(VariantArgs a) {
          p += (int64_t)gridDim.x * blockDim.x) {
         int m, E;
         if (a.shortest && __ldg(a.lens + p) < a.shortest) continue;
+        if (a.left_out && a.count[p] != kLeftOut) continue;
         if (!variant_args(a, p, &m, &E)) continue;
         const int ns = 2 * E + 1;
         Cursor x;
@@ -558,7 +562,10 @@ extern "C" pf_status pf_filter_partitioned(pf_ctx *ctx, const pf_pairs *pairs,
     // Rows of long pairs (long_words): 16 lanes per group or one pair a thread.
     // 0.33M pairs of 1000 bp, a fifth accepted: E = 8, t = 8, y = 2 545 us in tiles,
     // 567 one by one; t = 32, y = 1 545 and 295; E = 22 586 and 1431, 586 and 821.
-    // Where lengths are not known, the tiles leave the long pairs to a second launch.
+    // Where lengths are not known, the tiles leave the long pairs to a launch
+    // beside them, or, where tiles of long pairs are faster than that (E = 20,
+    // t = 8, y = 2 (176): 100,000 of 1000 bp 225 us and 490), a few of them to one
+    // behind them.
     const int64_t words = row_words(a.pairs);
     const bool maybe = words >= long_words(E_max), rows = maybe && words < INT64_MAX;
     const bool tiles = !E && (n >= 150000 ? E_max >= 8 || cost >= 18 : E_max >= 8 && cost >= 56) &&
@@ -568,10 +575,12 @@ extern "C" pf_status pf_filter_partitioned(pf_ctx *ctx, const pf_pairs *pairs,
         // 16 below, where the length of one tile counts: 250 bp, E = 12, 60,000
         // pairs take 33 us with 16 lanes, 200,000 take 53 with four.
         const int lanes = n < 80000 || rows ? 16 : 4;
-        const bool skip = maybe && !rows;
+        LongPairs late;
+        late.on = maybe && !rows;
+        late.few = late.on && E_max >= 16 && cost >= 100;
+        const bool beside = late.on && !late.few;
         cudaStream_t side = ctx->side_streams[0];
-        if (skip) {
-            // beside the tiles: a long pair's latency is theirs as a whole
+        if (beside) {   // a long pair's latency is the tiles' as a whole
             cudaEventRecord(ctx->ev_fork, ctx->stream);
             cudaStreamWaitEvent(side, ctx->ev_fork, 0);
             a.shortest = 32 * (long_words(E_max) - 1) + 1;
@@ -579,13 +588,15 @@ extern "C" pf_status pf_filter_partitioned(pf_ctx *ctx, const pf_pairs *pairs,
                            "pf_filter_partitioned launch");
         }
         const pf_status st2 = ctx->cuda(
-            launch_submat_sliced(filter_args_of(a), t, y, lanes, skip, ctx->sms, ctx->stream),
+            launch_submat_sliced(filter_args_of(a), t, y, lanes, late, ctx->sms, ctx->stream),
             "pf_filter_partitioned launch");
-        if (skip) {
+        if (beside) {
             cudaEventRecord(ctx->ev_join[0], side);
             cudaStreamWaitEvent(ctx->stream, ctx->ev_join[0], 0);
         }
-        return st != PF_OK ? st : st2;
+        if (st != PF_OK || st2 != PF_OK) return st != PF_OK ? st : st2;
+        if (!late.few) return PF_OK;
+        a.left_out = true;
     }
     return ctx->cuda(launch_variant<PartitionedK>(a, ctx->sms, ctx->stream),
                      "pf_filter_partitioned launch");

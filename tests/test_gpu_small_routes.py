@@ -40,7 +40,7 @@ def test_one_threshold(pf, E, dec, n):  # noqa: F811
     compare(pf, dec, pairs, lens, None, E, n)
 
 
-@pytest.mark.parametrize("E,dec,n", [(8, 1, 174_999), (15, 1, 175_000), (12, 3, 99_999),
+@pytest.mark.parametrize("E,dec,n", [(8, 1, 174_999), (14, 1, 175_000), (15, 1, 99_999), (15, 1, 100_000), (12, 3, 99_999),
                                      (12, 3, 100_000), (25, 2, 174_999), (25, 2, 175_000),
                                      (15, 3, 10_000), (15, 3, 10_001), (25, 1, 40_000),
                                      (25, 1, 40_001)])
